@@ -124,6 +124,8 @@ fr_status resolve_bulb(fr::DevReq &R, const fr_bulb_params *P)
                          P->normal_mode, P->normal_h);
 }
 
+bool bulb_wild(const fr::DevReq &R);
+
 // camera, light, plane and (when out != NULL) the output buffers
 fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam, const fr_light *li,
                          const fr_image *out, bool need_out = true)
@@ -203,6 +205,7 @@ fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam
         R.plane_hat = f4(n);
     }
 
+    R.wild = R.kind == FR_KIND_BULB && bulb_wild(R);
     if (!need_out) return FR_OK;
     if (!out->rgba8 && !out->rgba && !out->depth && !out->saved && !out->stats && !out->trap)
         return fail(FR_EINVAL, "image has no output buffer");
@@ -218,6 +221,21 @@ fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam
     R.stats = out->stats;
     R.trap = reinterpret_cast<float4 *>(out->trap);
     return FR_OK;
+}
+
+// Whether some iterate of a Mandelbulb request could leave the float range (and
+// come back as an infinity or a NaN that the orbit goes on with): such requests
+// run the general step.  An iterate comes from one inside the bailout, or from
+// the start of the orbit, a point of the bounding sphere or a stencil tap, and
+// ends at most at r^n + |c|; the other conditions keep the rounding of a point's
+// position far below the bounding sphere's own size.
+bool bulb_wild(const fr::DevReq &R)
+{
+    const double bound = std::sqrt((double)R.bound_r2);
+    const double eye2 = (double)R.eye.x * R.eye.x + (double)R.eye.y * R.eye.y + (double)R.eye.z * R.eye.z;
+    const double start = 1.01 * bound + 2.0 * R.normal_h + 1.0;
+    const double top = std::fmax(std::sqrt((double)R.esc2), start);
+    return !(bound < 1e3 && eye2 < 1e8 && R.eps < 1e3f && R.normal_h < 1e3f && std::pow(top, R.power) < 1e15);
 }
 
 // lanes per pixel of the one-ray-per-thread kernels: the pixel's samples on
@@ -271,7 +289,7 @@ fr_status resolve_requests(const fr_request *reqs, int n_reqs, std::vector<DevRe
             g_err = "request " + std::to_string(i) + ": " + g_err;
             return st;
         }
-        count = count || q.out.stats != nullptr;
+        count = count || q.out.stats != nullptr || R.wild;
     }
     return FR_OK;
 }
@@ -341,13 +359,13 @@ static fr_status launch_single(const fr::DevReq &R, bool count, void *stream)
         A.total_units = ctas;
         A.refill_threshold = 1;
         A.queue = nullptr;
-        return launched(fr::launch_batch_plain(A, ctas, tu.plain_block, tu.plain_unroll, count, R.shading != 0,
+        return launched(fr::launch_batch_plain(A, ctas, tu.plain_block, tu.plain_unroll, count || R.wild, R.shading != 0,
                                                (cudaStream_t)stream));
     }
     fr::DevReq Q = R;
     Q.tile_order = tu.tile_order;
     set_lanes(Q, lanes_per_pixel(tu, R));
-    return launched(fr::launch_plain(Q, tu.plain_block, tu.plain_unroll, count, (cudaStream_t)stream));
+    return launched(fr::launch_plain(Q, tu.plain_block, tu.plain_unroll, count || Q.wild, (cudaStream_t)stream));
 }
 
 FR_API fr_status fr_render_julia(const fr_julia_params *params, const fr_plane *plane,

@@ -213,7 +213,8 @@ __device__ void pixel_grad_bulb(const BwdArgs &A, int px, int py, float gsum[11]
         return;
     }
     Counters cnt;
-    const float3 n = normal_at<1, 1, false, true>(R, x, rd, cnt);
+    for (int k = 0; k < kNStats; k++) cnt.v[k] = 0;
+    const float3 n = R.wild ? normal_at<1, 1, true, true>(R, x, rd, cnt) : normal_at<1, 1, false, true>(R, x, rd, cnt);
     const float ndl = dot3(n, L);
     const float act = ndl > 0.0f ? W * R.kd * vis : 0.0f;
     gsum[8] += act * (n.x - L.x * ndl) / A.light_norm;

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) plain_kernel(const __grid_constant__ DevR
     if (COUNT)
         for (int k = 0; k < kNStats; k++) cnt.v[k] = 0;
     shade_tile<KIND, U, COUNT, PHONG, BAN, LANES>(R, gtid >> 5, cnt);
-    if (COUNT) flush_counters(cnt, R.stats);
+    if (COUNT && R.stats) flush_counters(cnt, R.stats);
 }
 
 template <int KIND, int U, bool COUNT, bool PHONG = false, int BAN = 0, bool LANES = false>

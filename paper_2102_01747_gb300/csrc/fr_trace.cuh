@@ -20,7 +20,7 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
     bool hit = true;
     for (int i = 0; i < R.max_steps; i++) {
         int trips;
-        float d = de<KIND, U>(R, along(ro, rd, t), trips);
+        float d = de<KIND, U, !COUNT>(R, along(ro, rd, t), trips);
         steps++;
         if (COUNT) cnt.v[kStatOrbit] += trips;
         if (d < R.eps) break;
@@ -63,7 +63,7 @@ __device__ __forceinline__ float3 normal_at(const DevReq &R, float3 x, float3 rd
     float3 g = v3(0.0f, 0.0f, 0.0f);
     for (int k = 0; k < taps; k++) {
         int trips;
-        const float d = de<KIND, U>(R, tap_point(x, R.normal_mode, R.normal_h, k), trips);
+        const float d = de<KIND, U, !COUNT>(R, tap_point(x, R.normal_mode, R.normal_h, k), trips);
         tap_accum(g, R.normal_mode, R.normal_h, k, d);
         if (COUNT) cnt.v[kStatOrbit] += trips;
     }
