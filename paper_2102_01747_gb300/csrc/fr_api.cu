@@ -125,6 +125,7 @@ fr_status resolve_bulb(fr::DevReq &R, const fr_bulb_params *P)
 }
 
 bool bulb_wild(const fr::DevReq &R);
+void set_exit(fr::DevReq &R);
 
 // camera, light, plane and (when out != NULL) the output buffers
 fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam, const fr_light *li,
@@ -220,6 +221,7 @@ fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam
     R.saved = reinterpret_cast<float4 *>(out->saved);
     R.stats = out->stats;
     R.trap = reinterpret_cast<float4 *>(out->trap);
+    set_exit(R);
     return FR_OK;
 }
 
@@ -236,6 +238,99 @@ bool bulb_wild(const fr::DevReq &R)
     const double start = 1.01 * bound + 2.0 * R.normal_h + 1.0;
     const double top = std::fmax(std::sqrt((double)R.esc2), start);
     return !(bound < 1e3 && eye2 < 1e8 && R.eps < 1e3f && R.normal_h < 1e3f && std::pow(top, R.power) < 1e15);
+}
+
+// A lower bound on the distance estimate at every point with |x| >= r, in
+// exact arithmetic; 0 if none is found.  *steps counts the orbit steps after
+// which such an orbit has escaped (or max_iter).
+//
+// Both estimates are phi = |z| log|z| / (2 |z'|), |z'| growing per step by
+// p r^(p-1) (Julia) or to n r^(n-1) |z'| + 1 (Mandelbulb).  A step from radius r
+// ends at s r^p with s >= 1 - C / r^p, C = |c| (for the Mandelbulb c is the point
+// itself), so
+//   phi_{k+1} / phi_k >= s (1 + log s / (p log r)) / (1 + 1 / (n r^(n-1) |z'|)),
+// (the last factor for the Mandelbulb only), which grows with s, r and |z'|.
+// The slowest orbit r <- r^p - C from |x| = r therefore bounds every factor
+// from below, for that |x| and for all larger ones (for the Mandelbulb
+// C / r_k^n falls as |x| grows), and an orbit that escapes earlier leaves
+// factors < 1 out.
+double distance_bound(const fr::DevReq &R, double r, int *steps)
+{
+    const bool bulb = R.kind == FR_KIND_BULB;
+    const int p = R.power;
+    const double C = bulb ? r : std::sqrt((double)R.c.x * R.c.x + (double)R.c.y * R.c.y +
+                                          (double)R.c.z * R.c.z + (double)R.c.w * R.c.w);
+    double lr = std::log(r), phi = 0.5 * r * lr, dz = 1.0;
+    int k = 0;
+    while (k < R.max_iter) {
+        k++;
+        double rn1 = 1.0;
+        for (int j = 1; j < p; j++) rn1 *= r;
+        const double s = (1.0 - C / (rn1 * r)) * (1.0 - 1e-4);  // the slack covers the kernels' rounding
+        const double next = s * rn1 * r;
+        if (!(next > r)) return 0.0;
+        const double ls = std::log(s);
+        phi *= s * (1.0 + ls / (p * lr));
+        if (bulb) {
+            phi /= 1.0 + 1.0 / (p * rn1 * dz);
+            dz = p * rn1 * dz + 1.0;
+        }
+        lr = p * lr + ls;
+        r = next;
+        if (r * r > (double)R.esc2) break;
+    }
+    *steps = k;
+    return phi > 0.0 ? phi : 0.0;
+}
+
+// The ball of exit_t: the first of a few radii from the smallest that can
+// escape upwards whose bound is well above eps (the kernels' float distance is
+// within 1e-3 of the exact one, relative) and outside which at most half the
+// step cap is needed to cross the bounding sphere, summed over shells of the
+// outside.  No ball (exit_r2 = 0) for extreme parameters, where float
+// distances could overflow or positions round coarsely.
+void set_exit(fr::DevReq &R)
+{
+    R.exit_r2 = 0.0f;
+    R.exit_steps = 0;
+    const bool bulb = R.kind == FR_KIND_BULB;
+    const double bound = std::sqrt((double)R.bound_r2);
+    const double eye2 = (double)R.eye.x * R.eye.x + (double)R.eye.y * R.eye.y + (double)R.eye.z * R.eye.z;
+    if (!(bound < 16.0) || !(eye2 < 256.0)) return;
+    const int p = R.power;
+    const double C = std::sqrt((double)R.c.x * R.c.x + (double)R.c.y * R.c.y + (double)R.c.z * R.c.z +
+                               (double)R.c.w * R.c.w);
+    // smallest radius that the slowest orbit leaves upwards
+    const double crit = bulb     ? std::exp2(1.0 / (p - 1))
+                        : p == 2 ? 0.5 + std::sqrt(0.25 + C)
+                                 : 1.0 + C / 2.0;  // r^3 - C >= r from here on
+    // largest |z| and |z'| the kernels can meet outside the ball
+    const double top = std::fmax(std::fmax(std::sqrt((double)R.esc2), std::hypot(bound, (double)R.slice_w)), 1.0);
+    const double cmax = bulb ? bound : C;
+    if (!((std::pow(top, p) + cmax) < 1e15)) return;
+    const double grow = bulb ? p * std::pow(top, p - 1) + 1.0 : p * p * std::pow(top, 2 * (p - 1));
+    static const double kScale[] = {1.01, 1.02, 1.04, 1.07, 1.12, 1.2, 1.35, 1.6};
+    for (double scale : kScale) {
+        const double r0 = crit * scale;
+        if (!(r0 < bound)) return;
+        int n = 0;
+        const double d0 = distance_bound(R, r0, &n);
+        if (!(d0 > 2.0 * R.eps && d0 > 1e-3) || !(n * std::log10(grow) < 30.0)) continue;
+        // crossing the shells r0 < |x| <= bound takes at most this many steps: in the shell from
+        // a to b at most 2 sqrt(b^2 - a^2) of any line, each step at least min(bound at a, max_step)
+        double steps = 2.0, a = r0, da = d0;
+        while (a < bound) {
+            const double b = std::fmin(1.1 * a, bound);
+            steps += 2.0 * (std::sqrt(b * b - a * a) / (0.98 * std::fmin(da, (double)R.max_step)) + 1.0);
+            a = b;
+            da = std::fmax(da, distance_bound(R, a, &n));
+            if (!(steps < R.max_steps)) break;
+        }
+        if (steps > 0.5 * R.max_steps) continue;
+        R.exit_steps = (int)std::ceil(steps);
+        R.exit_r2 = (float)(r0 * r0 + 2e-3);  // the margin covers rounding of positions within the ranges above
+        return;
+    }
 }
 
 // lanes per pixel of the one-ray-per-thread kernels: the pixel's samples on

@@ -99,13 +99,14 @@ static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 // CTAs to SMs as they free up, so the requests' slow pixels overlap instead of
 // each launch waiting for its own.  tile_begin of request r (in CTAs) is kept
 // in reqs[r].unit_begin.
-// Always compiled with the Mandelbulb's analytic normal (out of line), and held to 72
-// registers (at most 256 threads per block, as fr_set_tuning enforces): left
-// to itself the compiler takes 80, with which the 64-request mixed batch runs
-// 36.0 ms against 33.3 (64 registers: 33.5).  fr_render_* can also launch it
-// with one request (fr_tuning.single_kernel = 2, autotuned).
+// Always compiled with the Mandelbulb's analytic normal (out of line), and held to 80
+// registers (at most 256 threads per block, as fr_set_tuning enforces): with
+// marches that end at the ball the 64-request mixed batch runs 21.6 ms in 80
+// registers, 21.9 in 72, 22.0 in 88 and 24.3 in 64, 64 thumbnails 1.37, 1.46,
+// 1.37 and 1.6 ms.  fr_render_* can also launch it with one request
+// (fr_tuning.single_kernel = 2, autotuned).
 template <int U, bool COUNT, bool PHONG, bool LANES = false>
-__global__ void __maxnreg__(72) batch_plain_kernel(const __grid_constant__ BatchArgs A)
+__global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ BatchArgs A)
 {
     const int warps = blockDim.x >> 5;
     const long long cta = blockIdx.x;
@@ -146,7 +147,7 @@ static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int 
 // increasing order, so its request cursor only moves forward.  The pixels
 // are shade_tile's, so the images are the other schedules' bit for bit.
 template <int U, bool COUNT, bool PHONG, bool LANES = false>
-__global__ void __maxnreg__(72) batch_refill_kernel(const __grid_constant__ BatchArgs A)
+__global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ BatchArgs A)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;

@@ -10,7 +10,10 @@ namespace fr {
 
 // Sphere tracing (Listing "Julia Set ray cast"): from t0, d = DE(ro + t rd);
 // d < eps -> hit; t += min(d, max_step); t > t1 -> miss; running out of steps
-// inside the interval is reported as a hit at the current t.
+// inside the interval is reported as a hit at the current t.  The march ends as
+// a miss as soon as the ray has left the fractal's ball (exit_t) with steps
+// enough in hand to reach t1: the same outcome, without the distances on the
+// way out (the counting kernels take them, for their counters).
 template <int KIND, int U, bool COUNT>
 __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, float t0, float t1,
                                       float &t_out, int &steps_out, Counters &cnt, int slot)
@@ -18,17 +21,31 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
     float t = t0;
     int steps = 0;
     bool hit = true;
-    for (int i = 0; i < R.max_steps; i++) {
-        int trips;
-        float d = de<KIND, U, !COUNT>(R, along(ro, rd, t), trips);
-        steps++;
-        if (COUNT) cnt.v[kStatOrbit] += trips;
-        if (d < R.eps) break;
-        t = march_step(t, d, R.max_step);
-        if (t > t1) {
-            hit = false;
-            break;
+    float t_end = t1;
+    if (!COUNT) {
+        t_end = exit_t(R, ro, rd, t1);
+        if (t > t_end) {
+            if (R.exit_steps <= R.max_steps) return false;
+            t_end = t1;
         }
+    }
+    for (;;) {
+        while (steps < R.max_steps) {
+            int trips;
+            float d = de<KIND, U, !COUNT>(R, along(ro, rd, t), trips);
+            steps++;
+            if (COUNT) cnt.v[kStatOrbit] += trips;
+            if (d < R.eps) break;
+            t = march_step(t, d, R.max_step);
+            if (t > t_end) {
+                hit = false;
+                break;
+            }
+        }
+        // out of the ball too close to the step cap: on to t1 itself
+        if (COUNT || hit || t > t1 || steps + R.exit_steps <= R.max_steps) break;
+        t_end = t1;
+        hit = true;
     }
     if (COUNT) cnt.v[slot] += steps;
     t_out = t;
