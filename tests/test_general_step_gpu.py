@@ -27,9 +27,10 @@ def both(scene, **kw):
 
 @pytest.mark.parametrize("n", range(2, 17))
 @pytest.mark.parametrize("phong", [False, True])
-def test_every_power(n, phong):
+@pytest.mark.parametrize("algebraic", [False, True])
+def test_every_power(n, phong, algebraic):
     s = W.bulb_1080p(7 * n, 131, 93)
-    s.update(n=n, max_iter=6 + n, normal_mode=("tetra", "central", "analytic")[n % 3])
+    s.update(n=n, algebraic=algebraic, max_iter=6 + n, normal_mode=("tetra", "central", "analytic")[n % 3])
     s["camera"]["spp"] = (1, 2, 3, 4)[n % 4]
     both(W.phong(s) if phong else s)
 
@@ -40,6 +41,7 @@ def test_bailouts(n, bailout):
     s = W.bulb_1080p(3, 65, 47)
     s.update(n=n, bailout=bailout, max_iter=9)
     both(s)
+    both(dict(s, algebraic=True))
 
 
 @pytest.mark.parametrize("change", [dict(bound_radius=0.5), dict(bound_radius=50.0), dict(bound_radius=1e5),
@@ -60,6 +62,7 @@ def test_axis_and_origin():
             s.update(n=n, plane={"n": (0.0, 1.0, 0.0), "o": 0.0}, eps=1e-6)
             s["camera"].update(eye=eye, up=up, target=(0.0, 0.0, -1.0) if eye == (0.0, 0.0, 0.0) else (0.0, 0.0, 0.0))
             both(s)
+            both(dict(s, algebraic=True))
 
 
 def test_batch_with_an_overflowing_request():
