@@ -47,6 +47,7 @@ cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cud
         if (R.kind == 0)
             return count ? launch_plain_t<0, 1, true, true>(R, block, s) : launch_plain_t<0, 1, false, true>(R, block, s);
         if (count) return launch_plain_t<1, 1, true, true>(R, block, s);
+        if (R.power == 8 && !R.bulb_alg) return launch_plain_t<3, 4, false, true>(R, block, s);
         return R.power == 8 ? launch_plain_t<2, 4, false, true>(R, block, s) : launch_plain_t<1, 4, false, true>(R, block, s);
     }
     if (count) return R.kind == 0 ? launch_plain_t<0, 1, true>(R, block, s)
@@ -56,6 +57,8 @@ cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cud
         if (unroll == 2) return launch_plain_t<0, 2, false>(R, block, s);
         return launch_plain_t<0, 1, false>(R, block, s);
     }
+    if (R.power == 8 && !R.bulb_alg)
+        return unroll == 4 ? launch_plain_t<3, 4, false>(R, block, s) : launch_plain_t<3, 2, false>(R, block, s);
     if (R.power == 8)
         return unroll == 4 ? launch_plain_t<2, 4, false>(R, block, s) : launch_plain_t<2, 2, false>(R, block, s);
     return unroll == 4 ? launch_plain_t<1, 4, false>(R, block, s) : launch_plain_t<1, 2, false>(R, block, s);

@@ -12,10 +12,12 @@ cudaError_t launch_plain_ban(const DevReq &R, int block, bool count, cudaStream_
 {
     if (R.shading) {
         if (count) return launch_plain_t<1, 1, true, true, true>(R, block, s);
+        if (R.power == 8 && !R.bulb_alg) return launch_plain_t<3, 4, false, true, true>(R, block, s);
         return R.power == 8 ? launch_plain_t<2, 4, false, true, true>(R, block, s)
                             : launch_plain_t<1, 4, false, true, true>(R, block, s);
     }
     if (count) return launch_plain_t<1, 1, true, false, true>(R, block, s);
+    if (R.power == 8 && !R.bulb_alg) return launch_plain_t<3, 2, false, false, true>(R, block, s);
     return R.power == 8 ? launch_plain_t<2, 2, false, false, true>(R, block, s)
                         : launch_plain_t<1, 1, false, false, true>(R, block, s);
 }

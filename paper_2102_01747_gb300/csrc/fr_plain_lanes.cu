@@ -31,6 +31,7 @@ cudaError_t launch_plain_lanes(const DevReq &R, int block, bool count, cudaStrea
         return count ? launch_plain_t<1, 1, true, true, false, true>(R, block, s)
                      : launch_plain_t<1, 1, false, true, false, true>(R, block, s);
     if (count) return launch_plain_t<1, 1, true, false, false, true>(R, block, s);
+    if (R.power == 8 && !R.bulb_alg) return launch_plain_t<3, 2, false, false, false, true>(R, block, s);
     return R.power == 8 ? launch_plain_t<2, 2, false, false, false, true>(R, block, s)
                         : launch_plain_t<1, 4, false, false, false, true>(R, block, s);
 }
