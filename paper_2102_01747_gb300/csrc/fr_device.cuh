@@ -555,7 +555,11 @@ __device__ __forceinline__ float bulb_dist_tame(const Orbit &o)
     return quot(mul(mul(0.25f, log_own(o.m)), root), fminf(o.dz, 8.507059e37f));
 }
 
-// whole-orbit DEs (one-ray-per-thread kernel); trips = orbit loop trips.  TAME:
+// Whole-orbit DEs (one-ray-per-thread kernel); trips = orbit loop trips.  The
+// loops test the escape and the cap in one condition at their end (max_iter >=
+// 1): one branch per step, where a break in a counted loop took two.  With
+// march()'s loop written the same way: 4K Julia frame 1.38 -> 1.35 ms, cubic
+// Julia 0.19 -> 0.18, n = 5 frame 0.68 -> 0.60, 64 thumbnails 1.37 -> 1.34 ms.  TAME:
 // the Mandelbulb's bulb_step_tame, for requests that are not R.wild
 template <int U>
 __device__ __forceinline__ float julia_de2(const float4 c, float slice_w, int max_iter, float esc2,
@@ -565,11 +569,10 @@ __device__ __forceinline__ float julia_de2(const float4 c, float slice_w, int ma
     julia_init(o, p, slice_w);
     int i = 0;
 #pragma unroll U
-    for (int k = 0; k < max_iter; k++) {
+    do {
         julia2_step(o, c);
         i++;
-        if (o.m > esc2) break;
-    }
+    } while (!(o.m > esc2) && i < max_iter);
     trips = i;
     return julia_dist(o);
 }
@@ -582,11 +585,10 @@ __device__ __forceinline__ float julia_de3(const float4 c, float slice_w, int ma
     julia_init(o, p, slice_w);
     int i = 0;
 #pragma unroll U
-    for (int k = 0; k < max_iter; k++) {
+    do {
         julia3_step(o, c);
         i++;
-        if (o.m > esc2) break;
-    }
+    } while (!(o.m > esc2) && i < max_iter);
     trips = i;
     return julia_dist(o);
 }
@@ -599,7 +601,7 @@ __device__ __forceinline__ float bulb_orbit(int n, int max_iter, float esc2, flo
     if (TAME) o.d = fr_rsqrt_seed(o.m);
     int i = 0;
 #pragma unroll U
-    for (int k = 0; k < max_iter; k++) {
+    do {
         if (TAME && alg)
             bulb_step_alg_tame(o, c, n);
         else if (TAME)
@@ -609,8 +611,7 @@ __device__ __forceinline__ float bulb_orbit(int n, int max_iter, float esc2, flo
         else
             bulb_step(o, c, n);
         i++;
-        if (o.m > esc2) break;
-    }
+    } while (!(o.m > esc2) && i < max_iter);
     trips = i;
     return TAME ? bulb_dist_tame(o) : bulb_dist(o);
 }
@@ -726,7 +727,7 @@ __device__ __forceinline__ float3 julia_analytic_grad(const DevReq &R, float3 x,
     float4 ty = make_float4(0.0f, 1.0f, 0.0f, 0.0f);
     float4 tz = make_float4(0.0f, 0.0f, 1.0f, 0.0f);
     int i = 0;
-    for (int k = 0; k < R.max_iter; k++) {
+    do {
         tangent_step(tx, o, R.power);
         tangent_step(ty, o, R.power);
         tangent_step(tz, o, R.power);
@@ -735,8 +736,7 @@ __device__ __forceinline__ float3 julia_analytic_grad(const DevReq &R, float3 x,
         else
             julia3_step(o, R.c);
         i++;
-        if (o.m > R.esc2) break;
-    }
+    } while (!(o.m > R.esc2) && i < R.max_iter);
     trips = i;
     return v3(fmaf(o.d, tx.w, fmaf(o.c, tx.z, fmaf(o.b, tx.y, mul(o.a, tx.x)))),
               fmaf(o.d, ty.w, fmaf(o.c, ty.z, fmaf(o.b, ty.y, mul(o.a, ty.x)))),
@@ -824,7 +824,7 @@ __device__ __forceinline__ float3 bulb_analytic_normal(const DevReq &R, int n, f
         float3 w = x;
         float3 d = v3(col == 0 ? 1.0f : 0.0f, col == 1 ? 1.0f : 0.0f, col == 2 ? 1.0f : 0.0f);
         i = 0;
-        for (int k = 0; k < R.max_iter; k++) {
+        do {
             i++;
             float ir;
             const float r = sqrt_rsqrt_own(dot3(w, w), ir);
@@ -858,8 +858,7 @@ __device__ __forceinline__ float3 bulb_analytic_normal(const DevReq &R, int n, f
             d = v3(col == 0 ? add(dP.x, 1.0f) : dP.x, col == 1 ? add(dP.y, 1.0f) : dP.y,
                    col == 2 ? add(dP.z, 1.0f) : dP.z);
             w = v3(add(P.x, x.x), add(P.y, x.y), add(P.z, x.z));
-            if (dot3(w, w) > R.esc2) break;
-        }
+        } while (!(dot3(w, w) > R.esc2) && i < R.max_iter);
         const float gk = dot3(w, d);
         if (col == 0) g.x = gk;
         else if (col == 1) g.y = gk;

@@ -104,7 +104,9 @@ static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 // marches that end at the ball the 64-request mixed batch runs 21.6 ms in 80
 // registers, 21.9 in 72, 22.0 in 88 and 24.3 in 64, 64 thumbnails 1.37, 1.46,
 // 1.37 and 1.6 ms.  fr_render_* can also launch it with one request
-// (fr_tuning.single_kernel = 2, autotuned).
+// (fr_tuning.single_kernel = 2, autotuned).  The Mandelbulb's orbit loop is
+// unrolled twice as deep as the Julia set's (as in fr_plain.cu): at plain_unroll 1
+// 64 thumbnails take 1.34 ms with the loop rolled, 1.31 at depth 2, 1.38 at 4.
 template <int U, bool COUNT, bool PHONG, bool LANES = false>
 __global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ BatchArgs A)
 {
@@ -126,7 +128,7 @@ __global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ Batch
     if (R.kind == 0)
         shade_tile<0, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     else
-        shade_tile<1, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
+        shade_tile<1, 2 * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     if (COUNT && R.stats) flush_counters(cnt, R.stats);
 }
 
@@ -173,7 +175,7 @@ __global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ Batc
         if (R.kind == 0)
             shade_tile<0, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
         else
-            shade_tile<1, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
+            shade_tile<1, 2 * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     }
     if (COUNT && A.reqs[lo].stats) flush_counters(cnt, A.reqs[lo].stats);
 }

@@ -13,7 +13,8 @@ namespace fr {
 // inside the interval is reported as a hit at the current t.  The march ends as
 // a miss as soon as the ray has left the fractal's ball (exit_t) with steps
 // enough in hand to reach t1: the same outcome, without the distances on the
-// way out (the counting kernels take them, for their counters).
+// way out (the counting kernels take them, for their counters).  One condition
+// ends the loop (see the whole-orbit DEs).
 template <int KIND, int U, bool COUNT>
 __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, float t0, float t1,
                                       float &t_out, int &steps_out, Counters &cnt, int slot)
@@ -30,20 +31,24 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
         }
     }
     for (;;) {
-        while (steps < R.max_steps) {
+        bool going;
+        do {
             int trips;
-            float d = de<KIND, U, !COUNT>(R, along(ro, rd, t), trips);
+            const float d = de<KIND, U, !COUNT>(R, along(ro, rd, t), trips);
             steps++;
             if (COUNT) cnt.v[kStatOrbit] += trips;
-            if (d < R.eps) break;
-            t = march_step(t, d, R.max_step);
-            if (t > t_end) {
-                hit = false;
-                break;
-            }
-        }
+            const bool on = !(d < R.eps);
+            const float next = march_step(t, d, R.max_step);
+            t = on ? next : t;
+            hit = !(on && t > t_end);
+            going = on && hit && steps < R.max_steps;
+        } while (going);
         // out of the ball too close to the step cap: on to t1 itself
         if (COUNT || hit || t > t1 || steps + R.exit_steps <= R.max_steps) break;
+        if (steps == R.max_steps) {
+            hit = true;
+            break;
+        }
         t_end = t1;
         hit = true;
     }
