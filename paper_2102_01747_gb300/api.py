@@ -130,6 +130,12 @@ def current_stream(device=None):
     return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
 
 
+def scene_structs(scene: dict):
+    """The C structs of one scene: parameters (Julia or Mandelbulb), plane, camera, light."""
+    prm = julia_params(scene) if scene["kind"] == "julia" else bulb_params(scene)
+    return prm, plane_struct(scene), camera_struct(scene), light_struct(scene)
+
+
 def render(scene: dict, out: dict | None = None, stream=None, **alloc) -> dict:
     """Render one scene with the one-ray-per-thread kernel; returns the output
     tensors (allocated with alloc_image(**alloc) unless `out` is given)."""
@@ -137,13 +143,8 @@ def render(scene: dict, out: dict | None = None, stream=None, **alloc) -> dict:
         out = alloc_image(scene, **alloc)
     img = image_struct(out)
     s = stream if stream is not None else current_stream()
-    if scene["kind"] == "julia":
-        st = F.fr_render_julia(julia_params(scene), plane_struct(scene), camera_struct(scene),
-                               light_struct(scene), img, s)
-    else:
-        st = F.fr_render_mandelbulb(bulb_params(scene), plane_struct(scene), camera_struct(scene),
-                                    light_struct(scene), img, s)
-    F.check(st)
+    call = F.fr_render_julia if scene["kind"] == "julia" else F.fr_render_mandelbulb
+    F.check(call(*scene_structs(scene), img, s))
     return out
 
 

@@ -19,54 +19,67 @@ plane and the light (fr_render_backward_mandelbulb; the fractal has no c).
 """
 from __future__ import annotations
 
-import copy
-
 import torch
 
 from . import _ffi as F
 from . import api
 
 
-def _scene_with(scene, c, plane_n, plane_o, light_dir):
-    s = copy.deepcopy(scene)
-    s["c"] = tuple(float(v) for v in c.detach().cpu().tolist())
-    s["plane"] = {"n": tuple(float(v) for v in plane_n.detach().cpu().tolist()),
-                  "o": float(plane_o.detach().cpu().reshape(-1)[0])}
-    s["light"]["dir"] = tuple(float(v) for v in light_dir.detach().cpu().tolist())
-    return s
+def _scene_with(scene, plane_n, plane_o, light_dir, **fields):
+    """A copy of `scene` with the differentiable inputs' values; what stays the
+    same is shared, since the scene is only read until its C structs are made."""
+    plane = {"n": tuple(plane_n.detach().cpu().tolist()), "o": plane_o.detach().cpu().reshape(-1).tolist()[0]}
+    light = dict(scene["light"], dir=tuple(light_dir.detach().cpu().tolist()))
+    return dict(scene, plane=plane, light=light, **fields)
+
+
+def _forward(ctx, s, inputs):
+    """Renders s and keeps for the backward pass its structs (the same ones the
+    adjoint takes: the scene may change in between) and the saved hit state."""
+    out = api.alloc_image(s, rgba8=False, rgba=True, depth=True, saved=True)
+    ctx.structs = api.scene_structs(s)
+    call = F.fr_render_julia if s["kind"] == "julia" else F.fr_render_mandelbulb
+    F.check(call(*ctx.structs, api.image_struct(out), api.current_stream()))
+    ctx.save_for_backward(out["saved"])
+    ctx.in_dev = tuple(v.device for v in inputs)
+    return out["rgba"], out["depth"]
+
+
+def _backward(ctx, call, d_rgba, d_depth):
+    """The 11-vector of the adjoint `call`."""
+    (saved,) = ctx.saved_tensors
+    grad = torch.zeros(11, dtype=torch.float32, device=saved.device)
+    d_rgba = (torch.zeros_like(saved) if d_rgba is None else d_rgba).float().contiguous()
+    dd = None
+    if d_depth is not None:
+        dd = torch.nan_to_num(d_depth.float(), nan=0.0, posinf=0.0, neginf=0.0).contiguous()
+    ws = backward_workspace(saved.device)
+    F.check(call(*ctx.structs, saved.data_ptr(), d_rgba.data_ptr(), None if dd is None else dd.data_ptr(),
+                 grad.data_ptr(), ws.data_ptr(), ws.numel() * ws.element_size(), api.current_stream(saved.device)))
+    return grad
+
+
+def _parts(grad, bounds, devices):
+    """Slices of grad on their inputs' devices; inputs that all live elsewhere on
+    one device are served by one copy (each copy to the host waits for the GPU)."""
+    if len(set(devices)) == 1 and devices[0] != grad.device:
+        grad = grad.to(devices[0])
+        return [grad[a:b].clone() for a, b in bounds]
+    return [grad[a:b].to(d) for (a, b), d in zip(bounds, devices)]
 
 
 class JuliaRender(torch.autograd.Function):
     @staticmethod
     def forward(ctx, c, plane_n, plane_o, light_dir, scene):
-        s = _scene_with(scene, c, plane_n, plane_o, light_dir)
+        s = _scene_with(scene, plane_n, plane_o, light_dir, c=tuple(c.detach().cpu().tolist()))
         if s["kind"] != "julia" or s["camera"]["spp"] != 1:
             raise ValueError("the differentiable render takes a Julia scene with spp = 1")
-        out = api.render(s, rgba8=False, rgba=True, depth=True, saved=True)
-        ctx.scene = s
-        ctx.save_for_backward(out["saved"])
-        ctx.dev = out["rgba"].device
-        ctx.in_dev = (c.device, plane_n.device, plane_o.device, light_dir.device)
-        return out["rgba"], out["depth"]
+        return _forward(ctx, s, (c, plane_n, plane_o, light_dir))
 
     @staticmethod
     def backward(ctx, d_rgba, d_depth):
-        (saved,) = ctx.saved_tensors
-        s = ctx.scene
-        grad = torch.zeros(11, dtype=torch.float32, device=ctx.dev)
-        d_rgba = (torch.zeros_like(saved) if d_rgba is None else d_rgba).float().contiguous()
-        dd = None
-        if d_depth is not None:
-            dd = torch.nan_to_num(d_depth.float(), nan=0.0, posinf=0.0, neginf=0.0).contiguous()
-        ws = backward_workspace(ctx.dev)
-        st = F.fr_render_backward_ws(api.julia_params(s), api.plane_struct(s), api.camera_struct(s),
-                                     api.light_struct(s), saved.data_ptr(), d_rgba.data_ptr(),
-                                     None if dd is None else dd.data_ptr(), grad.data_ptr(),
-                                     ws.data_ptr(), ws.numel() * ws.element_size(),
-                                     api.current_stream(ctx.dev))
-        F.check(st)
-        dc, dn, do, dl = ctx.in_dev
-        return grad[0:4].to(dc), grad[4:7].to(dn), grad[7:8].to(do), grad[8:11].to(dl), None
+        grad = _backward(ctx, F.fr_render_backward_ws, d_rgba, d_depth)
+        return (*_parts(grad, ((0, 4), (4, 7), (7, 8), (8, 11)), ctx.in_dev), None)
 
 
 def julia_render(scene, c, plane_n, plane_o, light_dir):
@@ -79,28 +92,15 @@ class BulbRender(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, plane_n, plane_o, light_dir, scene):
-        s = copy.deepcopy(scene)
-        s["plane"] = {"n": tuple(float(v) for v in plane_n.detach().cpu().tolist()),
-                      "o": float(plane_o.detach().cpu().reshape(-1)[0])}
-        s["light"]["dir"] = tuple(float(v) for v in light_dir.detach().cpu().tolist())
+        s = _scene_with(scene, plane_n, plane_o, light_dir)
         if s["kind"] != "bulb" or s["camera"]["spp"] != 1:
             raise ValueError("the differentiable Mandelbulb render takes a Mandelbulb scene with spp = 1")
-        out = api.render(s, rgba8=False, rgba=True, depth=True, saved=True)
-        ctx.scene = s
-        ctx.save_for_backward(out["saved"])
-        ctx.in_dev = (plane_n.device, plane_o.device, light_dir.device)
-        return out["rgba"], out["depth"]
+        return _forward(ctx, s, (plane_n, plane_o, light_dir))
 
     @staticmethod
     def backward(ctx, d_rgba, d_depth):
-        (saved,) = ctx.saved_tensors
-        d_rgba = (torch.zeros_like(saved) if d_rgba is None else d_rgba).float().contiguous()
-        dd = None
-        if d_depth is not None:
-            dd = torch.nan_to_num(d_depth.float(), nan=0.0, posinf=0.0, neginf=0.0).contiguous()
-        grad = backward_raw(ctx.scene, saved, d_rgba, dd, workspace=backward_workspace(saved.device))
-        dn, do, dl = ctx.in_dev
-        return grad[4:7].to(dn), grad[7:8].to(do), grad[8:11].to(dl), None
+        grad = _backward(ctx, F.fr_render_backward_mandelbulb, d_rgba, d_depth)
+        return (*_parts(grad, ((4, 7), (7, 8), (8, 11)), ctx.in_dev), None)
 
 
 def bulb_render(scene, plane_n, plane_o, light_dir):
