@@ -71,9 +71,22 @@ __device__ __forceinline__ void shade_tile(const DevReq &R, long long tile, Coun
 }
 
 // BAN: compiled with the Mandelbulb's analytic normal (normal_at; 1 inline,
-// 2 out of line)
+// 2 out of line).
+// Register caps (at most 256 threads per block, as fr_set_tuning enforces):
+// given only the block size the compiler keeps to 73 registers and orders the
+// orbit step so that a warp waits on its own chain.  Measured at 64, 72, 80, 96
+// and 112 registers: the 1080p frame 0.69, 0.64, 0.61, 0.59, 0.60 ms, n = 6 at
+// 640x360 0.43, 0.41, 0.39, 0.37, 0.40, the 160x90 thumbnail 0.26, 0.21, 0.18,
+// 0.18, 0.18; Phong at 1080p 1.12, 1.04, 1.00, 0.98, 0.96 ms; 4K with 4 samples on
+// lanes 5.72, 5.66, 5.54, 5.59, 5.69.  The Julia set's kernels need 64.
+template <bool PHONG, bool LANES>
+constexpr int plain_registers()
+{
+    return LANES ? 80 : PHONG ? 112 : 96;
+}
+
 template <int KIND, int U, bool COUNT, bool PHONG, int BAN, bool LANES = false>
-__global__ void __launch_bounds__(256) plain_kernel(const __grid_constant__ DevReq R)
+__global__ void __maxnreg__((plain_registers<PHONG, LANES>())) plain_kernel(const __grid_constant__ DevReq R)
 {
     const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     Counters cnt;
