@@ -315,18 +315,14 @@ __device__ __forceinline__ float bulb_angles(float3 w, float ir, float nf, float
 
 // r^k for an integer 0 <= k < 16 by binary exponentiation (each product
 // rounded once, so r^7 carries at most 4 roundings).  Unrolled over the four
-// bits of k with the products selected, not branched on: the same products in
-// the same order as the loop over k's bits (res starts at 1, and 1 * b is b
-// exactly), without its data-dependent branches.
+// bits of k, which are uniform over the warp: each decides a product.
 __device__ __forceinline__ float ipow(float r, int k)
 {
-    float res = 1.0f, b = r;
-#pragma unroll
-    for (int bit = 0; bit < 4; bit++) {
-        const float p = mul(res, b);
-        res = ((k >> bit) & 1) ? p : res;
-        b = mul(b, b);
-    }
+    float res = (k & 1) ? r : 1.0f;
+    const float r2 = mul(r, r), r4 = mul(r2, r2), r8 = mul(r4, r4);
+    if (k & 2) res = mul(res, r2);
+    if (k & 4) res = mul(res, r4);
+    if (k & 8) res = mul(res, r8);
     return res;
 }
 
