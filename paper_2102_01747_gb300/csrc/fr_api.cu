@@ -520,14 +520,17 @@ FR_API fr_status fr_render_batch(const fr_request *reqs, int32_t n_reqs, void *w
     // costliest requests first: the cheap ones then fill in behind the costly
     // ones' slow pixels at the end of the launch (outputs travel with their
     // request).  Estimated cost: pixels x samples x orbit-iteration cap, x 6
-    // for the Mandelbulb (its step is about six Julia steps of instructions),
-    // x 1.4 with shadow rays.  Measured on 64 mixed requests: 32.6 ms against
-    // 33.1 ms ordered by pixels alone.
+    // for the Mandelbulb (its step is about six Julia steps of instructions), x 4
+    // and x 3 for the powers 2 and 3, whose sets reach out to radius 2 and take
+    // 380 and 350 iterations per pixel against about 100 for the others, x 1.4
+    // with shadow rays.  Measured without and with the powers' factors: 64 mixed
+    // requests 21.5 and 21.4 ms, 64 thumbnails 1.27 and 1.21 ms.
     std::vector<int> order((size_t)n_reqs);
     for (int i = 0; i < n_reqs; i++) order[(size_t)i] = i;
     auto cost = [&](int i) {
         const fr::DevReq &R = all[(size_t)i];
-        return (double)R.n_units * R.spp * R.max_iter * (R.kind == FR_KIND_BULB ? 6.0 : 1.0) *
+        const double bulb = R.power == 2 ? 24.0 : R.power == 3 ? 18.0 : 6.0;
+        return (double)R.n_units * R.spp * R.max_iter * (R.kind == FR_KIND_BULB ? bulb : 1.0) *
                (R.shadows ? 1.4 : 1.0);
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost(a) > cost(b); });
