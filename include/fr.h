@@ -202,8 +202,8 @@ typedef struct {
 /* Launch shapes; the autotuner writes them, every later call reads them. */
 typedef struct {
     int32_t plain_block;         /* threads per block of the one-ray-per-thread kernel (32..256, x32) */
-    int32_t plain_unroll;        /* orbit-loop unroll depth: 1, 2 or 4 (a single Mandelbulb
-                                    request takes at least 2)                         */
+    int32_t plain_unroll;        /* orbit-loop unroll depth: 1, 2 or 4 (a single
+                                    request takes at least 2)                     */
     int32_t persist_block;       /* threads per block of the persistent kernel          */
     int32_t persist_ctas_per_sm; /* resident CTAs per SM; 0 = as many as fit            */
     int32_t refill_threshold;    /* refill a warp once this many lanes are idle (1..32) */

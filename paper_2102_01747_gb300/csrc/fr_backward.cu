@@ -51,7 +51,7 @@ __device__ __forceinline__ float4 jt_cube(float4 z, float4 yb)
                        s * z.z + f * yb.z, s * z.w + f * yb.w);
 }
 
-// d(p) with d d / d p (gx) and d d / d c (gc) by reverse mode; d as in julia_de2/3
+// d(p) with d d / d p (gx) and d d / d c (gc) by reverse mode; d as in julia_de
 template <int P>
 __device__ float julia_de_grad(const DevReq &R, float3 p, float3 &gx, float4 &gc)
 {

@@ -557,34 +557,80 @@ __device__ __forceinline__ float bulb_dist_tame(const Orbit &o)
 // march()'s loop written the same way: 4K Julia frame 1.38 -> 1.35 ms, cubic
 // Julia 0.19 -> 0.18, n = 5 frame 0.68 -> 0.60, 64 thumbnails 1.37 -> 1.34 ms.  TAME:
 // the Mandelbulb's bulb_step_tame, for requests that are not R.wild
-template <int U>
-__device__ __forceinline__ float julia_de2(const float4 c, float slice_w, int max_iter, float esc2,
-                                           float3 p, int &trips)
+// The Julia set's step is short (36 cycles of dependent operations), and a test
+// of the escape after every step costs as much again.  So the orbit takes STEPS
+// steps per test (1 in the counting kernels): the distance needs only m and
+// |z'|, and where a step before the last ends the orbit its own are kept and what
+// was computed after it is thrown away.  Measured at 1, 2 and 4 steps: 256x256
+// 0.094, 0.075, 0.070 ms (its warps run almost alone, so the branch counts most),
+// 1001x667 of degree 3 0.18, 0.16, 0.17, the 4K frame 1.36, 1.32, 1.45.
+template <int P>
+__device__ __forceinline__ void julia_step(Orbit &o, const float4 c)
 {
-    Orbit o;
-    julia_init(o, p, slice_w);
-    int i = 0;
-#pragma unroll U
-    do {
+    if (P == 2)
         julia2_step(o, c);
-        i++;
-    } while (!(o.m > esc2) && i < max_iter);
-    trips = i;
-    return julia_dist(o);
+    else
+        julia3_step(o, c);
 }
 
-template <int U>
-__device__ __forceinline__ float julia_de3(const float4 c, float slice_w, int max_iter, float esc2,
-                                           float3 p, int &trips)
+template <int P, int U, int STEPS>
+__device__ __forceinline__ float julia_de(const float4 c, float slice_w, int max_iter, float esc2, float3 p,
+                                          int &trips)
 {
+    static_assert(STEPS == 1 || STEPS == 2 || STEPS == 4, "steps per test");
     Orbit o;
     julia_init(o, p, slice_w);
     int i = 0;
+    bool going;
+    if constexpr (STEPS == 1) {
 #pragma unroll U
-    do {
-        julia3_step(o, c);
-        i++;
-    } while (!(o.m > esc2) && i < max_iter);
+        do {
+            julia_step<P>(o, c);
+            i++;
+        } while (!(o.m > esc2) && i < max_iter);
+    } else if constexpr (STEPS == 2) {
+        float m1, dz1;
+        bool end1;
+#pragma unroll U
+        do {
+            julia_step<P>(o, c);
+            m1 = o.m;
+            dz1 = o.dz;
+            i += 2;
+            end1 = m1 > esc2 || i > max_iter;
+            julia_step<P>(o, c);
+            going = !end1 && !(o.m > esc2) && i < max_iter;
+        } while (going);
+        if (end1) {
+            o.m = m1;
+            o.dz = dz1;
+        }
+    } else {
+        float m1, dz1, m2, dz2, m3, dz3;
+        bool end1, end2, end3;
+#pragma unroll U
+        do {
+            julia_step<P>(o, c);
+            m1 = o.m;
+            dz1 = o.dz;
+            julia_step<P>(o, c);
+            m2 = o.m;
+            dz2 = o.dz;
+            julia_step<P>(o, c);
+            m3 = o.m;
+            dz3 = o.dz;
+            i += 4;
+            end1 = m1 > esc2 || i - 3 >= max_iter;
+            end2 = m2 > esc2 || i - 2 >= max_iter;
+            end3 = m3 > esc2 || i - 1 >= max_iter;
+            julia_step<P>(o, c);
+            going = !(end1 || end2 || end3) && !(o.m > esc2) && i < max_iter;
+        } while (going);
+        if (end1 || end2 || end3) {
+            o.m = end1 ? m1 : end2 ? m2 : m3;
+            o.dz = end1 ? dz1 : end2 ? dz2 : dz3;
+        }
+    }
     trips = i;
     return julia_dist(o);
 }
@@ -632,14 +678,17 @@ __device__ __forceinline__ float bulb_de(int n, int max_iter, float esc2, float3
 // whose power is 8 (the kernel then holds no code for other powers), 3 the same
 // without the trig-free form.  Less code is fewer waits for instructions: the
 // 1080p frame 0.65 ms as KIND 2, 0.63 as 3, the 160x90 thumbnail 0.23 and 0.21 ms.  TAME false
-// runs the general Mandelbulb step: the counting kernels do, and requests with
-// R.wild are launched on them.
+// runs the general Mandelbulb step and single Julia steps: the counting kernels
+// do, and requests with R.wild are launched on them.
+constexpr int kJuliaQuads = 8;  // U of the Julia kernels that take four steps per test
+
 template <int KIND, int U, bool TAME>
 __device__ __forceinline__ float de(const DevReq &R, float3 p, int &trips)
 {
     if (KIND == 0) {
-        if (R.power == 2) return julia_de2<U>(R.c, R.slice_w, R.max_iter, R.esc2, p, trips);
-        return julia_de3<U>(R.c, R.slice_w, R.max_iter, R.esc2, p, trips);
+        constexpr int steps = !TAME ? 1 : U == kJuliaQuads ? 4 : 2, unroll = U == kJuliaQuads ? 1 : U;
+        if (R.power == 2) return julia_de<2, unroll, steps>(R.c, R.slice_w, R.max_iter, R.esc2, p, trips);
+        return julia_de<3, unroll, steps>(R.c, R.slice_w, R.max_iter, R.esc2, p, trips);
     }
     if (KIND == 3) return bulb_orbit<U, TAME>(8, R.max_iter, R.esc2, p, 0, trips);
     return bulb_de<U, TAME>(KIND == 2 ? 8 : R.power, R.max_iter, R.esc2, p, R.bulb_alg, trips);

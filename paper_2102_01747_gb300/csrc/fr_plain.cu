@@ -32,20 +32,20 @@ cudaError_t launch_batch_refill(const BatchArgs &A, int block, int unroll, bool 
 
 // Phong requests run the Phong-capable instantiation at one unroll depth;
 // Mandelbulb requests of the paper's power 8 (not counting) an instantiation for
-// that power.  The Mandelbulb's loops take at least two steps per trip, the
-// Phong ones four: a step is long enough to leave the loop's own branch and
+// that power.  The loops take at least two steps per trip, the
+// Mandelbulb's Phong ones four: a step is long enough to leave the loop's own branch and
 // counter waiting on its chain, and unrolled the next step's start overlaps them.
-// Measured at depths 1, 2 and 4: the 1080p frame 0.70, 0.64, 0.66 ms, n = 6 at
+// Measured at depths 1, 2 and 4, the Mandelbulb: the 1080p frame 0.70, 0.64, 0.66 ms, n = 6 at
 // 640x360 0.52, 0.47, 0.50 ms, n = 3 at 1283x723 0.95, 0.94, 0.92 ms; Phong at
-// 1080p 1.06, 1.07, 1.02 ms, at 320x180 0.38, 0.39, 0.34 ms.  The Julia step is
-// short and best rolled (4K 1.38 ms against 1.42).
+// 1080p 1.06, 1.07, 1.02 ms, at 320x180 0.38, 0.39, 0.34 ms.  The Julia set's
+// depth counts pairs of steps (julia_de): the 4K frame 1.335, 1.320, 1.329 ms.
 cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cudaStream_t s)
 {
     if (R.spl > 1) return launch_plain_lanes(R, block, count, s);
     if (R.kind == 1 && R.normal_mode == 2) return launch_plain_ban(R, block, count, s);
     if (R.shading) {
         if (R.kind == 0)
-            return count ? launch_plain_t<0, 1, true, true>(R, block, s) : launch_plain_t<0, 1, false, true>(R, block, s);
+            return count ? launch_plain_t<0, 1, true, true>(R, block, s) : launch_plain_t<0, 2, false, true>(R, block, s);
         if (count) return launch_plain_t<1, 1, true, true>(R, block, s);
         if (R.power == 8 && !R.bulb_alg) return launch_plain_t<3, 4, false, true>(R, block, s);
         return R.power == 8 ? launch_plain_t<2, 4, false, true>(R, block, s) : launch_plain_t<1, 4, false, true>(R, block, s);
@@ -53,9 +53,10 @@ cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cud
     if (count) return R.kind == 0 ? launch_plain_t<0, 1, true>(R, block, s)
                                   : launch_plain_t<1, 1, true>(R, block, s);
     if (R.kind == 0) {
-        if (unroll == 4) return launch_plain_t<0, 4, false>(R, block, s);
-        if (unroll == 2) return launch_plain_t<0, 2, false>(R, block, s);
-        return launch_plain_t<0, 1, false>(R, block, s);
+        // an image whose warps run almost alone (at most four per scheduler) is best
+        // served by the fewest tests
+        if (plain_tiles(R) <= 2432) return launch_plain_t<0, kJuliaQuads, false>(R, block, s);
+        return unroll == 4 ? launch_plain_t<0, 4, false>(R, block, s) : launch_plain_t<0, 2, false>(R, block, s);
     }
     if (R.power == 8 && !R.bulb_alg)
         return unroll == 4 ? launch_plain_t<3, 4, false>(R, block, s) : launch_plain_t<3, 2, false>(R, block, s);

@@ -67,3 +67,13 @@ def test_small_exponents():
         s = W.bulb_1080p(40, 97, 71)
         s.update(n=n, bound_radius=2.5, plane=None)
         both(s)
+
+
+@pytest.mark.parametrize("max_iter", [1, 2, 3, 4, 5, 6, 9, 11])
+@pytest.mark.parametrize("p", [2, 3])
+@pytest.mark.parametrize("size", [(97, 71), (412, 395)])
+def test_julia_steps_per_escape_test(size, p, max_iter):
+    # small images take four orbit steps per escape test, larger ones two, the counting kernels one
+    s = W.resized(julia((-0.3, 0.5, 0.3, 0.1), p=p, max_iter=max_iter), *size)
+    both(s)
+    both(W.phong(dict(s, normal_mode="tetra")))
