@@ -478,9 +478,11 @@ __device__ __forceinline__ void bulb_step_alg(Orbit &o, float3 cpt, int n)
 
 // The same step (same bits) for requests that are not R.wild: as
 // bulb_step_tame, without the branches on r > 0 and rho > 0 and with the root's
-// seed carried in o.d; the powers of both unit complex numbers are taken at once
-// as packed pairs (of the polar and the azimuth angle).  The trig-free 1080p
-// frame takes 0.45 ms against 0.51 with bulb_step_alg.
+// seed carried in o.d; for n = 8 the powers of both unit complex numbers are
+// taken at once as packed pairs (of the polar and the azimuth angle).  The trig-free 1080p
+// frame takes 0.45 ms against 0.51 with bulb_step_alg.  Other powers keep
+// cpow_int's scalar products and selects, and their loop stays rolled: n = 6 at
+// 1283x723 0.71 ms, in packed pairs 0.77 (0.81 rolled), as before the change 0.82.
 __device__ __forceinline__ void bulb_step_alg_tame(Orbit &o, float3 cpt, int n)
 {
     const float nf = (float)n;
@@ -505,22 +507,14 @@ __device__ __forceinline__ void bulb_step_alg_tame(Orbit &o, float3 cpt, int n)
             s = mul2(cs, dup2(2.0f));
             ns = mul2(cs, dup2(-2.0f));
         }
-    } else {  // cpow_int
-        f32x2 ac = dup2(1.0f), as = dup2(0.0f);
-#pragma unroll
-        for (int bit = 0; bit < 5; bit++) {
-            const f32x2 tc = fma2(ac, c, mul2(as, ns));
-            const f32x2 ts = fma2(ac, s, mul2(as, c));
-            const bool take = (n >> bit) & 1;
-            ac = take ? tc : ac;
-            as = take ? ts : as;
-            const f32x2 cs = mul2(c, s);
-            c = fma2(c, c, mul2(s, ns));
-            s = mul2(cs, dup2(2.0f));
-            ns = mul2(cs, dup2(-2.0f));
-        }
-        c = ac;
-        s = as;
+    } else {
+        float c0, c1, s0, s1, p0, p1, q0, q1;
+        unpack2(c, c0, c1);
+        unpack2(s, s0, s1);
+        cpow_int(c0, s0, n, p0, q0);
+        cpow_int(c1, s1, n, p1, q1);
+        c = pack2(p0, p1);
+        s = pack2(q0, q1);
     }
     float cb, ca, sb, sa;
     unpack2(c, cb, ca);
@@ -668,7 +662,7 @@ __device__ __forceinline__ float bulb_de(int n, int max_iter, float esc2, float3
 {
     if (alg) {
         if (n == 8) return bulb_orbit<U, TAME>(8, max_iter, esc2, c, 1, trips);
-        return bulb_orbit<U, TAME>(n, max_iter, esc2, c, 1, trips);
+        return bulb_orbit<1, TAME>(n, max_iter, esc2, c, 1, trips);  // cpow_int is long: rolled
     }
     if (n == 8) return bulb_orbit<U, TAME>(8, max_iter, esc2, c, 0, trips);
     return bulb_orbit<U, TAME>(n, max_iter, esc2, c, 0, trips);
