@@ -369,12 +369,11 @@ __device__ __forceinline__ void bulb_step(Orbit &o, float3 cpt, int n)
 //
 // The step is bound by issue slots where the GPU is full and by its chain of
 // dependent operations at a frame's end, when the slowest rays run alone.
-// Against bulb_step: the 1080p frame (camera at a random azimuth) 491 M warp
-// instructions against 387 M, 0.86 against 0.70 ms; a 160 x 90 thumbnail, one
-// warp per scheduler, 0.39 against 0.26 ms; the 4K frame with 4 samples 7.0
-// against 6.2 ms.  With the last five terms of the angles' polynomials packed as
-// well the thumbnail took 0.25 ms, but their pairs of constants took registers
-// or loads that slowed the 4K frame by 2 % and the mixed batch by 12 %.
+// In place of bulb_step: the 1080p frame (camera at a random azimuth) 0.85 ->
+// 0.71 ms, a 160 x 90 thumbnail, less than one warp per scheduler, 0.36 -> 0.25 ms,
+// the 4K frame with 4 samples 6.9 -> 6.4 ms (with all that came after, 0.59, 0.16
+// and 5.5 ms).  With the last five terms of the angles' polynomials packed as well
+// the pairs of constants take registers or loads: 4K 5.9 against 5.5 ms.
 __device__ __forceinline__ void bulb_step_tame(Orbit &o, float3 cpt, int n)
 {
     const float nf = (float)n;
