@@ -397,7 +397,7 @@ fr_status resolve_requests(const fr_request *reqs, int n_reqs, std::vector<DevRe
             g_err = "request " + std::to_string(i) + ": " + g_err;
             return st;
         }
-        count = count || q.out.stats != nullptr || R.wild;
+        count = count || q.out.stats != nullptr;
     }
     return FR_OK;
 }
@@ -467,7 +467,7 @@ static fr_status launch_single(const fr::DevReq &R, bool count, void *stream)
         A.total_units = ctas;
         A.refill_threshold = 1;
         A.queue = nullptr;
-        return launched(fr::launch_batch_plain(A, ctas, tu.plain_block, tu.plain_unroll, count || R.wild, R.shading != 0,
+        return launched(fr::launch_batch_plain(A, ctas, tu.plain_block, tu.plain_unroll, count, R.shading != 0,
                                                (cudaStream_t)stream));
     }
     fr::DevReq Q = R;

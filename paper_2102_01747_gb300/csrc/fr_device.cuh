@@ -667,12 +667,23 @@ __device__ __forceinline__ float bulb_de(int n, int max_iter, float esc2, float3
     return bulb_orbit<U, TAME>(n, max_iter, esc2, c, 0, trips);
 }
 
+// The general step out of line, for kernels that hold the other one too.
+static __device__ __noinline__ float bulb_de_general(int n, int max_iter, float esc2, float3 c, int alg, int *trips)
+{
+    int t;
+    const float d = bulb_de<1, false>(n, max_iter, esc2, c, alg, t);
+    *trips = t;
+    return d;
+}
+
 // KIND: 0 the Julia set, 1 the Mandelbulb, 2 the Mandelbulb of a request
 // whose power is 8 (the kernel then holds no code for other powers), 3 the same
 // without the trig-free form.  Less code is fewer waits for instructions: the
-// 1080p frame 0.65 ms as KIND 2, 0.63 as 3, the 160x90 thumbnail 0.23 and 0.21 ms.  TAME false
-// runs the general Mandelbulb step and single Julia steps: the counting kernels
-// do, and requests with R.wild are launched on them.
+// 1080p frame 0.65 ms as KIND 2, 0.63 as 3, the 160x90 thumbnail 0.23 and 0.21 ms.
+// 4 the Mandelbulb by the general step whether R.wild or not, 5 the Mandelbulb by
+// the step that the request needs (batch launches with wild requests in them).
+// TAME false runs the general Mandelbulb step and single Julia steps, as the
+// counting kernels do.
 constexpr int kJuliaQuads = 8;  // U of the Julia kernels that take four steps per test
 
 template <int KIND, int U, bool TAME>
@@ -684,6 +695,8 @@ __device__ __forceinline__ float de(const DevReq &R, float3 p, int &trips)
         return julia_de<3, unroll, steps>(R.c, R.slice_w, R.max_iter, R.esc2, p, trips);
     }
     if (KIND == 3) return bulb_orbit<U, TAME>(8, R.max_iter, R.esc2, p, 0, trips);
+    if (KIND == 4) return bulb_de<U, false>(R.power, R.max_iter, R.esc2, p, R.bulb_alg, trips);
+    if (KIND == 5 && R.wild) return bulb_de_general(R.power, R.max_iter, R.esc2, p, R.bulb_alg, &trips);
     return bulb_de<U, TAME>(KIND == 2 ? 8 : R.power, R.max_iter, R.esc2, p, R.bulb_alg, trips);
 }
 

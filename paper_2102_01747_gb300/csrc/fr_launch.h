@@ -72,6 +72,13 @@ cudaError_t launch_batch_plain_lanes(const BatchArgs &A, long long ctas, int blo
 cudaError_t launch_batch_refill(const BatchArgs &A, int block, int unroll, bool count, bool phong, cudaStream_t s);
 cudaError_t launch_batch_refill_lanes(const BatchArgs &A, int block, bool count, bool phong, cudaStream_t s);
 
+// the same two for a launch without counters in which some request is wild; bulb: the
+// Mandelbulb's KIND (4 or 5), lanes: some request has spl > 1
+cudaError_t launch_batch_plain_wild(const BatchArgs &A, long long ctas, int block, bool phong, bool lanes, int bulb,
+                                    cudaStream_t s);
+cudaError_t launch_batch_refill_wild(const BatchArgs &A, int block, bool phong, bool lanes, int bulb,
+                                     cudaStream_t s);
+
 // lane-state-machine forward kernel without the queue: one pixel per lane, all tiles launched
 cudaError_t launch_lanes(const BatchArgs &A, int block, int unroll, bool count, bool phong, cudaStream_t s);
 

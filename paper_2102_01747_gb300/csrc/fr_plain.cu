@@ -5,13 +5,38 @@
 
 namespace fr {
 
+// Of a batch launch: whether some request has its samples on adjacent lanes, and the
+// Mandelbulb's KIND: 1, or with wild requests among them 5, which holds both steps,
+// or 4 where the wild ones are at least half of the Mandelbulbs' work (pixels x
+// samples x iteration cap), since the general step serves every request.  64 mixed
+// requests with the Mandelbulbs' bailouts at 10^(22/n), as 4 and as 5: one wild request
+// 21.5 and 20.6 ms, a quarter of them 21.2 and 20.8, half 20.4 and 20.8, 15 of 16 20.1 and
+// 20.9 (none wild 20.2); on the counting kernels 22.3, 22.0, 21.1 and 20.7.
+static void traits(const BatchArgs &A, bool &lanes, int &bulb)
+{
+    double wild = 0.0, all = 0.0;
+    lanes = false;
+    for (int i = 0; i < A.n_reqs; i++) {
+        const DevReq &R = A.reqs[i];
+        lanes = lanes || R.spl > 1;
+        if (R.kind != 1) continue;
+        const double work = (double)R.n_units * R.spp * R.max_iter;
+        all += work;
+        if (R.wild) wild += work;
+    }
+    bulb = wild == 0.0 ? 1 : wild < 0.5 * all ? 5 : 4;
+}
+
 // phong: some request of the launch uses Phong shading (the Phong-capable code
 // then serves every request of the launch, at unroll 1)
 cudaError_t launch_batch_plain(const BatchArgs &A, long long ctas, int block, int unroll, bool count,
                                bool phong, cudaStream_t s)
 {
-    for (int i = 0; i < A.n_reqs; i++)
-        if (A.reqs[i].spl > 1) return launch_batch_plain_lanes(A, ctas, block, count, phong, s);
+    bool lanes;
+    int bulb;
+    traits(A, lanes, bulb);
+    if (bulb != 1 && !count) return launch_batch_plain_wild(A, ctas, block, phong, lanes, bulb, s);
+    if (lanes) return launch_batch_plain_lanes(A, ctas, block, count, phong, s);
     if (phong) return count ? launch_batch_plain_t<1, true, true>(A, ctas, block, s)
                             : launch_batch_plain_t<1, false, true>(A, ctas, block, s);
     if (count) return launch_batch_plain_t<1, true, false>(A, ctas, block, s);
@@ -21,8 +46,11 @@ cudaError_t launch_batch_plain(const BatchArgs &A, long long ctas, int block, in
 
 cudaError_t launch_batch_refill(const BatchArgs &A, int block, int unroll, bool count, bool phong, cudaStream_t s)
 {
-    for (int i = 0; i < A.n_reqs; i++)
-        if (A.reqs[i].spl > 1) return launch_batch_refill_lanes(A, block, count, phong, s);
+    bool lanes;
+    int bulb;
+    traits(A, lanes, bulb);
+    if (bulb != 1 && !count) return launch_batch_refill_wild(A, block, phong, lanes, bulb, s);
+    if (lanes) return launch_batch_refill_lanes(A, block, count, phong, s);
     if (phong) return count ? launch_batch_refill_t<1, true, true>(A, block, s)
                             : launch_batch_refill_t<1, false, true>(A, block, s);
     if (count) return launch_batch_refill_t<1, true, false>(A, block, s);

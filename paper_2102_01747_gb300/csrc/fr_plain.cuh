@@ -120,8 +120,16 @@ static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 // (fr_tuning.single_kernel = 2, autotuned).  The Mandelbulb's orbit loop is
 // unrolled twice as deep as the Julia set's (as in fr_plain.cu): at plain_unroll 1
 // 64 thumbnails take 1.34 ms with the loop rolled, 1.31 at depth 2, 1.38 at 4.
-template <int U, bool COUNT, bool PHONG, bool LANES = false>
-__global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ BatchArgs A)
+// BULB is the Mandelbulb's KIND; the general step alone (4) runs rolled in 72 registers
+// (64 mixed requests, all Mandelbulbs wild: 22.2 ms, unrolled in 80 22.9).
+template <int BULB>
+constexpr int batch_registers()
+{
+    return BULB == 4 ? 72 : 80;
+}
+
+template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+__global__ void __maxnreg__((batch_registers<BULB>())) batch_plain_kernel(const __grid_constant__ BatchArgs A)
 {
     const int warps = blockDim.x >> 5;
     const long long cta = blockIdx.x;
@@ -141,14 +149,14 @@ __global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ Batch
     if (R.kind == 0)
         shade_tile<0, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     else
-        shade_tile<1, 2 * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
+        shade_tile<BULB, (BULB == 4 ? 1 : 2) * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     if (COUNT && R.stats) flush_counters(cnt, R.stats);
 }
 
-template <int U, bool COUNT, bool PHONG, bool LANES = false>
+template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int block, cudaStream_t s)
 {
-    batch_plain_kernel<U, COUNT, PHONG, LANES><<<(unsigned)ctas, block, 0, s>>>(A);
+    batch_plain_kernel<U, COUNT, PHONG, LANES, BULB><<<(unsigned)ctas, block, 0, s>>>(A);
     return cudaGetLastError();
 }
 
@@ -161,8 +169,8 @@ static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int 
 // reqs[r].unit_begin holds request r's first tile.  A warp's tiles come in
 // increasing order, so its request cursor only moves forward.  The pixels
 // are shade_tile's, so the images are the other schedules' bit for bit.
-template <int U, bool COUNT, bool PHONG, bool LANES = false>
-__global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ BatchArgs A)
+template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+__global__ void __maxnreg__((batch_registers<BULB>())) batch_refill_kernel(const __grid_constant__ BatchArgs A)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -188,24 +196,24 @@ __global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ Batc
         if (R.kind == 0)
             shade_tile<0, U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
         else
-            shade_tile<1, 2 * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
+            shade_tile<BULB, (BULB == 4 ? 1 : 2) * U, COUNT, PHONG, 2, LANES>(R, tile, cnt);
     }
     if (COUNT && A.reqs[lo].stats) flush_counters(cnt, A.reqs[lo].stats);
 }
 
-template <int U, bool COUNT, bool PHONG, bool LANES = false>
+template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 static cudaError_t launch_batch_refill_t(const BatchArgs &A, int block, cudaStream_t s)
 {
     int dev = 0, sms = 0, fit = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, batch_refill_kernel<U, COUNT, PHONG, LANES>, block,
-                                                           0)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, batch_refill_kernel<U, COUNT, PHONG, LANES, BULB>,
+                                                           block, 0)) != cudaSuccess)
         return e;
     if (fit < 1) return cudaErrorInvalidConfiguration;
     if ((e = cudaMemsetAsync(A.queue, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
-    batch_refill_kernel<U, COUNT, PHONG, LANES><<<sms * fit, block, 0, s>>>(A);
+    batch_refill_kernel<U, COUNT, PHONG, LANES, BULB><<<sms * fit, block, 0, s>>>(A);
     return cudaGetLastError();
 }
 
