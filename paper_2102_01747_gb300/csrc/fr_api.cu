@@ -474,7 +474,7 @@ static fr_status launch_single(const fr::DevReq &R, bool count, void *stream)
     Q.tile_order = tu.tile_order;
     set_lanes(Q, lanes_per_pixel(tu, R));
     if (tu.sample_lanes && R.spp == 1 && R.kind == FR_KIND_BULB && !R.shading) set_lanes(Q, idle_lanes(R));
-    return launched(fr::launch_plain(Q, tu.plain_block, tu.plain_unroll, count || Q.wild, (cudaStream_t)stream));
+    return launched(fr::launch_plain(Q, tu.plain_block, tu.plain_unroll, count, (cudaStream_t)stream));
 }
 
 FR_API fr_status fr_render_julia(const fr_julia_params *params, const fr_plane *plane,

@@ -51,6 +51,9 @@ cudaError_t launch_backward(const BwdArgs &A, cudaStream_t s);
 // one-ray-per-thread forward kernel for one request
 cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cudaStream_t s);
 
+// the same for a wild request without counters
+cudaError_t launch_plain_wild(const DevReq &R, int block, cudaStream_t s);
+
 // one-ray-per-thread kernel over A.n_reqs requests in one launch; reqs[r].unit_begin
 // holds request r's first CTA, `ctas` the grid size; phong: some request uses
 // Phong shading

@@ -69,6 +69,7 @@ cudaError_t launch_batch_refill(const BatchArgs &A, int block, int unroll, bool 
 // depth counts pairs of steps (julia_de): the 4K frame 1.335, 1.320, 1.329 ms.
 cudaError_t launch_plain(const DevReq &R, int block, int unroll, bool count, cudaStream_t s)
 {
+    if (R.wild && !count) return launch_plain_wild(R, block, s);
     if (R.spl > 1) return launch_plain_lanes(R, block, count, s);
     if (R.kind == 1 && R.normal_mode == 2) return launch_plain_ban(R, block, count, s);
     if (R.shading) {

@@ -120,16 +120,11 @@ static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 // (fr_tuning.single_kernel = 2, autotuned).  The Mandelbulb's orbit loop is
 // unrolled twice as deep as the Julia set's (as in fr_plain.cu): at plain_unroll 1
 // 64 thumbnails take 1.34 ms with the loop rolled, 1.31 at depth 2, 1.38 at 4.
-// BULB is the Mandelbulb's KIND; the general step alone (4) runs rolled in 72 registers
-// (64 mixed requests, all Mandelbulbs wild: 22.2 ms, unrolled in 80 22.9).
-template <int BULB>
-constexpr int batch_registers()
-{
-    return BULB == 4 ? 72 : 80;
-}
-
+// BULB is the Mandelbulb's KIND; the general step alone (4) stays rolled (one such request
+// as single_kernel 2: 0.83 ms in 72 registers, 0.81 in 80, 0.80 unrolled in 80; 64 mixed requests,
+// all Mandelbulbs wild: 24.3, 24.6, 24.4 ms; 64 of sides 64..512 as batch_kernel 1: 4.28, 4.19, 4.23).
 template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
-__global__ void __maxnreg__((batch_registers<BULB>())) batch_plain_kernel(const __grid_constant__ BatchArgs A)
+__global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ BatchArgs A)
 {
     const int warps = blockDim.x >> 5;
     const long long cta = blockIdx.x;
@@ -170,7 +165,7 @@ static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int 
 // increasing order, so its request cursor only moves forward.  The pixels
 // are shade_tile's, so the images are the other schedules' bit for bit.
 template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
-__global__ void __maxnreg__((batch_registers<BULB>())) batch_refill_kernel(const __grid_constant__ BatchArgs A)
+__global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ BatchArgs A)
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;

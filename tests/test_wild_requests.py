@@ -46,3 +46,18 @@ def test_only_the_launch_with_the_wild_request_changes():
     scenes[7].update(n=8, max_iter=100, bailout=1e4)  # costliest: in the first launch
     first, second, third = D.launches(scenes, batch=True)
     assert first[1][-1] == 5 and second == third and second[1][-1] == 1
+
+
+@pytest.mark.parametrize("normal_mode", ["tetra", "analytic"])
+@pytest.mark.parametrize("phong", [False, True])
+@pytest.mark.parametrize("spp", [1, 4])
+def test_single_wild_request(spp, phong, normal_mode):
+    s = wild(640, 360, normal_mode=normal_mode)
+    s["camera"]["spp"] = spp
+    s = W.phong(s) if phong else s
+    ban = int(normal_mode == "analytic")
+    assert D.launches(s) == [("plain_kernel", (4, 2, 0, int(phong), ban, int(spp == 4)))]
+    ((name, args),) = D.launches(s, stats=True)
+    assert name == "plain_kernel" and args[2] == 1
+    ((name, args),) = D.launches(s, tuning=dict(single_kernel=2, plain_unroll=1))
+    assert name == "batch_plain_kernel" and args == (1, 0, int(phong), int(spp == 4), 4)

@@ -71,3 +71,25 @@ def test_batch_with_wild_requests(batch_kernel, spp, phong):
         torch.cuda.synchronize()
     for i, (o, r) in enumerate(zip(outs, refs)):
         same(o, r, i)
+
+
+@pytest.mark.parametrize("normal_mode", ["tetra", "central", "analytic"])
+@pytest.mark.parametrize("phong", [False, True])
+@pytest.mark.parametrize("n", [2, 3, 8, 16])
+def test_single_wild_requests(n, phong, normal_mode):
+    import torch
+    from paper_2102_01747_gb300 import api
+
+    for i, (w, h) in enumerate(((61, 45), (258, 151))):  # spare lanes, one lane per pixel
+        for spp in (1, 3, 4):
+            s = W.bulb_1080p(9 * n, w, h)
+            s.update(n=n, bailout=10.0 ** (22.0 / n), max_iter=5 + i, normal_mode=normal_mode, algebraic=spp == 3)
+            s["camera"]["spp"] = spp
+            s = W.phong(s) if phong else s
+            ref = general(s)
+            for kernel in (0, 2):
+                with tuned(single_kernel=kernel):
+                    out = api.render(s, **OUTS)
+                    torch.cuda.synchronize()
+                same(out, ref, (w, spp, kernel))
+
