@@ -1,5 +1,5 @@
-"""Mandelbulb requests whose iterates may overflow (large bailouts and radii) take
-the general orbit step.  Which kernels such calls launch: none that counts, and
+"""Mandelbulb requests whose iterates may overflow (large bailouts and radii: r^n up to
+1e19 keeps |w|^2 finite) take the general orbit step.  Which kernels such calls launch: none that counts, and
 none that a request beside them would not have."""
 import pytest
 
@@ -61,3 +61,22 @@ def test_single_wild_request(spp, phong, normal_mode):
     assert name == "plain_kernel" and args[2] == 1
     ((name, args),) = D.launches(s, tuning=dict(single_kernel=2, plain_unroll=1))
     assert name == "batch_plain_kernel" and args == (1, 0, int(phong), int(spp == 4), 4)
+
+
+@pytest.mark.parametrize("n", range(2, 17))
+def test_limit(n):
+    limit = 1e19 ** (1.0 / n)
+    for field, value in (("bailout", limit), ("bound_radius", (limit - 1.0) / 1.01)):
+        for factor, general in ((0.999, False), (1.001, True)):
+            s = dict(W.bulb_1080p(10, 640, 360), n=n, **{field: value * factor})
+            ((name, args),) = D.launches(s)
+            if field == "bound_radius" and n < 7:
+                general = value * factor >= 1e3  # positions round too coarsely
+            assert (args[0] == 4) == general, (field, factor)
+
+
+def test_the_listings_bailout():
+    # |w|^2 > 256 ends the listing's orbit: the step without special paths for every power but 16
+    for n in range(2, 17):
+        ((name, args),) = D.launches(dict(W.bulb_1080p(10, 640, 360), n=n, bailout=16.0))
+        assert (args[0] == 4) == (n == 16)

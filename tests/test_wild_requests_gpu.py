@@ -93,3 +93,21 @@ def test_single_wild_requests(n, phong, normal_mode):
                     torch.cuda.synchronize()
                 same(out, ref, (w, spp, kernel))
 
+
+
+@pytest.mark.parametrize("n", range(2, 17))
+def test_both_steps_on_either_side_of_the_limit(n):
+    import torch
+    from paper_2102_01747_gb300 import api
+
+    limit = 1e19 ** (1.0 / n)
+    for factor in (0.5, 0.9999, 1.0001):
+        s = W.bulb_1080p(11 * n, 150, 110)
+        s.update(n=n, bailout=limit * factor, max_iter=9, algebraic=factor == 0.5)
+        s["camera"]["spp"] = 3  # one lane per pixel
+        far = dict(s, plane=None, bailout=2.0, bound_radius=min((limit - 1.0) / 1.01 * factor, 990.0), max_step=50.0)
+        for scene in (s, far, dict(s, algebraic=factor != 0.5)):
+            ref = general(scene)
+            out = api.render(scene, **OUTS)
+            torch.cuda.synchronize()
+            same(out, ref, (factor, scene["bound_radius"]))
