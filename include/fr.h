@@ -202,8 +202,14 @@ typedef struct {
 /* Launch shapes; the autotuner writes them, every later call reads them. */
 typedef struct {
     int32_t plain_block;         /* threads per block of the one-ray-per-thread kernel (32..256, x32) */
-    int32_t plain_unroll;        /* orbit-loop unroll depth: 1, 2 or 4 (a single
-                                    request takes at least 2)                     */
+    int32_t plain_unroll;        /* orbit-loop unroll depth: 1, 2 or 4.  Read by the batch
+                                    kernels of batch_kernel 1 and 2 and of single_kernel 2
+                                    (1 or 2; 4 as 1) where no request uses Phong shading,
+                                    lanes per sample or counters, and by single_kernel 0 (2
+                                    or 4; 1 as 2) for Lambert images on one lane per pixel,
+                                    but for small Julia images, and Mandelbulbs with the
+                                    analytic normal or iterates that may overflow; every
+                                    other kernel has one depth                     */
     int32_t persist_block;       /* threads per block of the persistent kernel          */
     int32_t persist_ctas_per_sm; /* resident CTAs per SM; 0 = as many as fit            */
     int32_t refill_threshold;    /* refill a warp once this many lanes are idle (1..32) */
@@ -231,6 +237,9 @@ typedef struct {
                                     covers 4 x 8 / spp pixels, whose jittered rays take
                                     nearly the same marches), 0 each lane runs its
                                     pixel's samples in turn (4 x 8 pixels per warp).
+                                    With spp 1 and single_kernel 0, 1 also gives the pixels
+                                    of Lambert Mandelbulbs of at most 1024 tiles (4 x 8
+                                    pixels each) 2, 4 or 8 lanes, of which one works.
                                     Same images bit for bit.                           */
 } fr_tuning;
 

@@ -13,7 +13,10 @@ For fr_render_batch (tune):
   persist_unroll     Julia orbit steps per scheduling round (the unroll depth)
 For one request through fr_render_julia / fr_render_mandelbulb (tune_single):
   single_kernel      0 the single-request kernel, 2 the batch kernel's code
-  plain_block, plain_unroll (orbit-loop unroll depth), tile_order and sample_lanes.
+  plain_block, tile_order
+  plain_unroll       orbit-loop unroll depth, where the request's kernel has more than one
+  sample_lanes       as above, and for small Lambert Mandelbulbs of one sample: spare lanes
+                     (1) or one pixel per lane (0)
 The search is coordinate descent from the current setting: each knob in turn is
 swept with the others fixed, each candidate timed with CUDA events (median of a
 few calls on the caller's scenes), and a candidate replaces the current
@@ -134,13 +137,37 @@ def tune_single(scene, reps: int = 9, passes: int = 1, space: dict | None = None
     candidate."""
     out = api.alloc_image(scene)
     apply({"single_kernel": 0 if start_kernel is None else start_kernel})
-    lanes = _sample_lanes_matter([scene])
-    return _descent(lambda: _time_single(scene, out, reps), space or SINGLE_SPACE,
-                    lambda k, c: k != "sample_lanes" or (lanes and c.get("single_kernel", 0) != 1), passes,
-                    log, margin)
+    return _descent(lambda: _time_single(scene, out, reps), space or SINGLE_SPACE, lambda k, c: True, passes, log,
+                    margin, lambda knob, cfg: _effect(scene, knob, cfg))
 
 
-def _descent(timer, space, in_use, passes, log, margin) -> dict:
+def _tiles(scene) -> int:
+    cam = scene["camera"]
+    return -(-cam["width"] // 4) * -(-cam["height"] // 8)
+
+
+def _effect(scene, knob: str, cfg: dict):
+    """What the knob's value in `cfg` comes to for one request: values of the same effect
+    launch the same kernel (the launchers' rules: launch_single, launch_plain)."""
+    kernel, cam = cfg["single_kernel"], scene["camera"]
+    bulb, phong = scene["kind"] == "bulb", scene["light"].get("shading", "lambert") == "phong"
+    spare = kernel == 0 and bulb and not phong and cam["spp"] == 1 and _tiles(scene) <= 1024
+    lanes = kernel != 1 and cfg["sample_lanes"] and (cam["spp"] in (2, 4, 8) or spare)
+    if knob == "sample_lanes":
+        return lanes
+    if knob == "plain_unroll":
+        fixed = phong or lanes or kernel == 1
+        if kernel == 0 and bulb:
+            fixed = fixed or scene["normal_mode"] == "analytic"
+        elif kernel == 0:
+            fixed = fixed or (_tiles(scene) <= 2432 and scene["max_iter"] > 2)
+        if fixed:
+            return 0
+        return (4 if cfg[knob] == 4 else 2) if kernel == 0 else (2 if cfg[knob] == 2 else 1)
+    return cfg[knob]
+
+
+def _descent(timer, space, in_use, passes, log, margin, effect=lambda knob, cfg: cfg[knob]) -> dict:
     best = current()
     best_ms = timer()
     trials = [dict(best, ms=best_ms)]
@@ -149,9 +176,9 @@ def _descent(timer, space, in_use, passes, log, margin) -> dict:
             if not in_use(knob, best):
                 continue
             for v in values:
-                if v == best[knob]:
-                    continue
                 cand = dict(best, **{knob: v})
+                if effect(knob, cand) == effect(knob, best):
+                    continue
                 apply(cand)
                 ms = timer()
                 trials.append(dict(cand, ms=ms))

@@ -83,8 +83,9 @@ struct __align__(16) DevReq {
     int shading;              // 0 Lambert, 1 Phong + reflection bounce
     int quad_store;           // rgba8 / depth rows may be written 4 pixels per 16-byte store
     int tile_order;           // order of the tiles over the grid (fr_tuning.tile_order)
-    int spl;                  // one-ray-per-thread kernels: lanes per pixel (1, or spp when the
-                              // pixel's samples run on adjacent lanes; fr_tuning.sample_lanes)
+    int spl;                  // one-ray-per-thread kernels: lanes per pixel (1; spp when the pixel's
+                              // samples run on adjacent lanes; 2, 4 or 8 with spp 1, the first of
+                              // them at work; fr_tuning.sample_lanes)
     int spl_log2;             // log2(spl)
     float exit_r2;        // squared radius of a ball around the fractal beyond which every distance
                           // exceeds eps (0: none known); see exit_t

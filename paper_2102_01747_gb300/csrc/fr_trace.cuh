@@ -267,8 +267,10 @@ __device__ __forceinline__ void render_pixel(const DevReq &R, int px, int py, Co
 
 // The same pixel, called by all 32 lanes of the warp together, with its spp
 // samples on R.spl adjacent lanes: sample k on the k-th when R.spl = spp (2, 4
-// or 8), all samples in turn on one lane when R.spl = 1 (requests of a batch
-// launch that some other request's spl > 1 put on this code).  With spl = spp
+// or 8), the one sample on the first when spp = 1 (small Mandelbulb images; the
+// others idle, so that a warp waits for fewer rays), all samples in turn on one lane
+// when R.spl = 1 (requests of a batch launch that some other request's spl > 1 put
+// on this code).  With spl = spp
 // the warp's 32 rays come from 32 / spp neighbouring pixels (a tile
 // 4 x 8 / spp pixels) whose samples are a fraction of a pixel apart, so they
 // take nearly the same march and orbit lengths and keep more lanes busy.  The

@@ -68,9 +68,10 @@ def _fake(scene, **want):
     return img
 
 
-def launches(scenes, batch=False, tuning=None, **want):
+def launches(scenes, batch=False, tuning=None, shapes=False, **want):
     """Kernels of one call on `scenes` (a scene, or a list of them for fr_render_batch) with
-    the tuning's fields replaced by `tuning`: a list of (name, template arguments)."""
+    the tuning's fields replaced by `tuning`: a list of (name, template arguments), with `shapes` also
+    (..., CTAs, threads per CTA)."""
     lib = load()
     want = want or dict(rgba8=True, depth=True)
     keep = F.fr_tuning()
@@ -95,4 +96,5 @@ def launches(scenes, batch=False, tuning=None, **want):
         assert st == F.FR_OK, lib.fr_last_error()
     finally:
         lib.fr_set_tuning(ctypes.byref(keep))
-    return [parse(line.split()[0]) for line in lib.fake_launches(1).decode().splitlines()]
+    lines = [line.split() for line in lib.fake_launches(1).decode().splitlines()]
+    return [(*parse(k), int(g), int(b)) if shapes else parse(k) for k, g, b in lines]
