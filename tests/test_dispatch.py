@@ -44,3 +44,16 @@ def test_the_tuner_times_each_kernel_once(monkeypatch):
                     cand = dict(base, **{knob: v})
                     differs = D.launches(s, tuning=cand, shapes=True) != D.launches(s, tuning=base, shapes=True)
                     assert (cand in trials[1:]) == differs, (s, knob, v)
+
+
+def test_kernel_scenes_reach_every_forward_kernel():
+    import kernel_scenes
+
+    reached = set()
+    for group in kernel_scenes.GROUPS.values():
+        for name, scenes, batch, tuning, stats in group():
+            want = dict(rgba8=True, depth=True, stats=stats)
+            reached.update(D.launches(scenes if batch else scenes[0], batch, tuning, **want))
+    forward = {k for k in D.kernels() if k[0] not in ("backward_kernel", "ffma_probe_kernel")}
+    assert reached <= forward
+    assert reached == forward, sorted(forward - reached)
