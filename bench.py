@@ -350,15 +350,21 @@ def max_over_ranks(torch, dist, seconds: float, device) -> float:
     return float(t.item())
 
 
-def count_scenes(api, torch, scenes):
-    """Counting-kernel pass (untimed): the FR_STAT_* counters of each scene."""
+def count_scenes(api, torch, scenes, to_end=False):
+    """Untimed pass: the FR_STAT_* counters of each scene, of the distances and orbit
+    iterations that the timed kernels evaluate (fr_work_probe), or to_end of marches to
+    the end of their interval (the counting kernels; the lane state machine's work)."""
     from paper_2102_01747_gb300 import _ffi as F
 
     per = []
     for s in scenes:
-        c = api.render(s, rgba8=False, depth=False, stats=True)
+        if to_end:
+            c = api.render(s, rgba8=False, depth=False, stats=True)["stats"]
+        else:
+            c = torch.zeros(F.FR_NSTATS, dtype=torch.int64, device="cuda")
+            F.check(F.fr_work_probe(api.request_struct(s, {}), c.data_ptr(), api.current_stream()))
         torch.cuda.synchronize()
-        per.append([int(v) for v in c["stats"].cpu().tolist()][:F.FR_NSTATS])
+        per.append([int(v) for v in c.cpu().tolist()][:F.FR_NSTATS])
     return per
 
 
@@ -458,7 +464,12 @@ def measure(args, torch, api, F, scenes, path, env, steps, warmup, clk_index=Non
         r = autotune.tune_single(scenes[0], reps=max(tune_reps, 3), space=space, start_kernel=args.single_kernel)
         tuning = {"config": r["config"], "search_ms": r["ms"], "trials": len(r["trials"]),
                   "trial_ms": [[{k: t[k] for k in space}, round(t["ms"], 4)] for t in r["trials"]]}
-    per = count_scenes(api, torch, scenes)
+    tu = F.fr_get_tuning()
+    if path == "plain":  # the kernel fr_render_* launches under the tuned single_kernel
+        kern = {0: "plain_kernel", 1: "persist_kernel", 2: "batch_plain_kernel"}[tu.single_kernel]
+    else:
+        kern = {0: "persist_kernel", 1: "batch_plain_kernel", 2: "batch_refill_kernel"}[tu.batch_kernel]
+    per = count_scenes(api, torch, scenes, to_end=kern == "persist_kernel")
     tot = _sum_counts(per)
     flops_ncu = sum(flops_per_iter(s) * c[5] for s, c in zip(scenes, per))
     flops_alg = sum(alg_flops(s, c) for s, c in zip(scenes, per))
@@ -473,11 +484,6 @@ def measure(args, torch, api, F, scenes, path, env, steps, warmup, clk_index=Non
         times, total_s, clk = time_steps(torch, step, steps, tstream, flush, dist,
                                          clk_index=clk_index if pth == path else None)
         results[pth] = {"times": times, "total_s": total_s, "clk": clk, "launches": step.launches()}
-    tu = F.fr_get_tuning()
-    if path == "plain":  # the kernel fr_render_* launches under the tuned single_kernel
-        kern = {0: "plain_kernel", 1: "persist_kernel", 2: "batch_plain_kernel"}[tu.single_kernel]
-    else:
-        kern = {0: "persist_kernel", 1: "batch_plain_kernel", 2: "batch_refill_kernel"}[tu.batch_kernel]
     main_r = results[path]
     return {"per": per, "counts": tot, "flops_ncu": flops_ncu, "flops_alg": flops_alg, "outs": outs,
             "results": results, "main": main_r, "kernel": kern, "tuning": tuning,
@@ -827,6 +833,7 @@ def main():
                    "parallelism": "replicas (one frame per rank)" if world > 1 else "single GPU"},
         "de_evals_per_s": des_of(counts) * args.steps * world / total_s,
         "orbit_iters_per_s": counts[5] * args.steps * world / total_s,
+        "counted": "distances and orbit iterations as the timed kernels evaluate them (fr_work_probe)",
         "per_step": {"rays": rays_per_step, "primary_rays": counts[0], "shadow_rays": counts[1],
                      "mirror_rays": counts[6], "de_calls": des_of(counts), "orbit_iters": counts[5]},
         "per_request": ([{"rays": rays_of(c), "de_calls": des_of(c), "orbit_iters": c[5]} for c in m["per"]]

@@ -377,6 +377,16 @@ FR_API fr_status fr_render_backward_ws(const fr_julia_params *params, const fr_p
 FR_API fr_status fr_ffma_probe(int32_t blocks, int32_t threads, int32_t iters, float *sink, void *stream);
 FR_API double fr_ffma_probe_flops(int32_t blocks, int32_t threads, int32_t iters);
 
+/* Diagnostic beside it, for the roofline's numerator: adds to `counters` (device,
+ * FR_NSTATS, 8-byte aligned) what the image kernels evaluate for one request.
+ * fr_image.stats counts marches to the end of their interval; the kernels that
+ * only render end a march once it has left a ball around the fractal outside
+ * which no distance is below eps, so their distances and orbit iterations are
+ * fewer.  The rays are the same.  request->out is not read.  (Not what
+ * single_kernel 1 and batch_kernel 0 evaluate: they march to the end.)
+ * Errors: FR_EINVAL, FR_ECUDA. */
+FR_API fr_status fr_work_probe(const fr_request *request, unsigned long long *counters, void *stream);
+
 /* Read / replace the process-wide launch shapes (checked; FR_EINVAL if out of range). */
 FR_API fr_status fr_get_tuning(fr_tuning *out);
 FR_API fr_status fr_set_tuning(const fr_tuning *t);

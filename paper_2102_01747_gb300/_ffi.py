@@ -97,6 +97,7 @@ SIGNATURES = {
                                         c_void_p, c_void_p, c_void_p, c_void_p, ctypes.c_size_t,
                                         c_void_p]),
     "fr_ffma_probe": (c_int32, [c_int32, c_int32, c_int32, c_void_p, c_void_p]),
+    "fr_work_probe": (c_int32, [ctypes.POINTER(fr_request), c_void_p, c_void_p]),
     "fr_ffma_probe_flops": (ctypes.c_double, [c_int32, c_int32, c_int32]),
     "fr_get_tuning": (c_int32, [ctypes.POINTER(fr_tuning)]),
     "fr_set_tuning": (c_int32, [ctypes.POINTER(fr_tuning)]),
@@ -193,6 +194,10 @@ def fr_render_backward_mandelbulb(params, plane, camera, light, saved, d_rgba, d
 
 def fr_ffma_probe(blocks, threads, iters, sink, stream=None):
     return load().fr_ffma_probe(int(blocks), int(threads), int(iters), sink, stream)
+
+
+def fr_work_probe(request, counters, stream=None):
+    return load().fr_work_probe(ctypes.byref(request), counters, stream)
 
 
 def fr_ffma_probe_flops(blocks, threads, iters) -> float:

@@ -52,7 +52,7 @@ __device__ __forceinline__ void tile_pixel(const DevReq &R, long long tile, int 
 // turn; LANES true: the samples of a pixel on R.spl adjacent lanes), called by
 // all 32 lanes of the warp; the packed colour and depth of finished pixels go
 // to the warp's quad store.
-template <int KIND, int U, bool COUNT, bool PHONG, int BAN, bool LANES>
+template <int KIND, int U, int COUNT, bool PHONG, int BAN, bool LANES>
 __device__ __forceinline__ void shade_tile(const DevReq &R, long long tile, Counters &cnt)
 {
     const int lane = threadIdx.x & 31;
@@ -85,7 +85,7 @@ constexpr int plain_registers()
     return LANES ? 80 : PHONG ? 112 : 96;
 }
 
-template <int KIND, int U, bool COUNT, bool PHONG, int BAN, bool LANES = false>
+template <int KIND, int U, int COUNT, bool PHONG, int BAN, bool LANES = false>
 __global__ void __maxnreg__((plain_registers<PHONG, LANES>())) plain_kernel(const __grid_constant__ DevReq R)
 {
     const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -96,7 +96,7 @@ __global__ void __maxnreg__((plain_registers<PHONG, LANES>())) plain_kernel(cons
     if (COUNT && R.stats) flush_counters(cnt, R.stats);
 }
 
-template <int KIND, int U, bool COUNT, bool PHONG = false, int BAN = 0, bool LANES = false>
+template <int KIND, int U, int COUNT, bool PHONG = false, int BAN = 0, bool LANES = false>
 static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 {
     const long long threads = plain_tiles(R) * 32;
@@ -123,7 +123,7 @@ static cudaError_t launch_plain_t(const DevReq &R, int block, cudaStream_t s)
 // BULB is the Mandelbulb's KIND; the general step alone (4) stays rolled (one such request
 // as single_kernel 2: 0.83 ms in 72 registers, 0.81 in 80, 0.80 unrolled in 80; 64 mixed requests,
 // all Mandelbulbs wild: 24.3, 24.6, 24.4 ms; 64 of sides 64..512 as batch_kernel 1: 4.28, 4.19, 4.23).
-template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+template <int U, int COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 __global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ BatchArgs A)
 {
     const int warps = blockDim.x >> 5;
@@ -148,7 +148,7 @@ __global__ void __maxnreg__(80) batch_plain_kernel(const __grid_constant__ Batch
     if (COUNT && R.stats) flush_counters(cnt, R.stats);
 }
 
-template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+template <int U, int COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int block, cudaStream_t s)
 {
     batch_plain_kernel<U, COUNT, PHONG, LANES, BULB><<<(unsigned)ctas, block, 0, s>>>(A);
@@ -164,7 +164,7 @@ static cudaError_t launch_batch_plain_t(const BatchArgs &A, long long ctas, int 
 // reqs[r].unit_begin holds request r's first tile.  A warp's tiles come in
 // increasing order, so its request cursor only moves forward.  The pixels
 // are shade_tile's, so the images are the other schedules' bit for bit.
-template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+template <int U, int COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 __global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ BatchArgs A)
 {
     const unsigned full = 0xffffffffu;
@@ -196,7 +196,7 @@ __global__ void __maxnreg__(80) batch_refill_kernel(const __grid_constant__ Batc
     if (COUNT && A.reqs[lo].stats) flush_counters(cnt, A.reqs[lo].stats);
 }
 
-template <int U, bool COUNT, bool PHONG, bool LANES = false, int BULB = 1>
+template <int U, int COUNT, bool PHONG, bool LANES = false, int BULB = 1>
 static cudaError_t launch_batch_refill_t(const BatchArgs &A, int block, cudaStream_t s)
 {
     int dev = 0, sms = 0, fit = 0;

@@ -1,5 +1,7 @@
-// fr_probe.cu -- the FP32 fused multiply-add throughput of the GPU the
-// library runs on: the denominator of the renderer's FP32 roofline.
+// fr_probe.cu -- the two sides of the renderer's FP32 roofline: the fused
+// multiply-add throughput of the GPU the library runs on (ffma_probe_kernel), and
+// the distances and orbit iterations that a request's image takes (fr_work_probe:
+// plain_kernel with kCountTaken).
 //
 // Every thread runs kChains independent chains x <- x * a + b, each link one
 // FFMA; kChains independent chains per thread and several warps per scheduler
@@ -7,11 +9,14 @@
 // issue rate.  a is just below 1 and b small, so the values stay finite; the
 // chains' sum is stored once per thread so that none of them is dead code.
 #include <cstdint>
+#include <vector>
 
 #include "../../include/fr.h"
+#include "fr_plain.cuh"
 
 namespace fr {
 fr_status set_error(fr_status st, const char *msg);
+fr_status resolve_requests(const fr_request *reqs, int n_reqs, std::vector<DevReq> &all, bool &count);
 }
 
 namespace {
@@ -56,6 +61,27 @@ FR_API fr_status fr_ffma_probe(int32_t blocks, int32_t threads, int32_t iters, f
     if (!sink || ((uintptr_t)sink % 4)) return fr::set_error(FR_EINVAL, "sink is NULL or misaligned");
     ffma_probe_kernel<<<blocks, threads, 0, (cudaStream_t)stream>>>(iters, 0.9999999f, 1e-7f, sink);
     const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return fr::set_error(FR_ECUDA, cudaGetErrorString(e));
+    fr::set_error(FR_OK, "");
+    return FR_OK;
+}
+
+FR_API fr_status fr_work_probe(const fr_request *request, unsigned long long *counters, void *stream)
+{
+    fr::NvtxRange range("fr_work_probe");
+    if (!request) return fr::set_error(FR_EINVAL, "request is NULL");
+    if (!counters) return fr::set_error(FR_EINVAL, "counters is NULL");
+    fr_request q = *request;
+    q.out = fr_image{};
+    q.out.stats = counters;
+    std::vector<fr::DevReq> all;
+    bool count = false;
+    const fr_status st = fr::resolve_requests(&q, 1, all, count);
+    if (st != FR_OK) return st;
+    // the Phong-capable code with the analytic normal serves every request
+    const cudaError_t e =
+        all[0].kind == 0 ? fr::launch_plain_t<0, 1, fr::kCountTaken, true, 1>(all[0], 128, (cudaStream_t)stream)
+                         : fr::launch_plain_t<1, 1, fr::kCountTaken, true, 1>(all[0], 128, (cudaStream_t)stream);
     if (e != cudaSuccess) return fr::set_error(FR_ECUDA, cudaGetErrorString(e));
     fr::set_error(FR_OK, "");
     return FR_OK;

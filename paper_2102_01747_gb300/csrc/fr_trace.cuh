@@ -8,14 +8,19 @@
 
 namespace fr {
 
+// COUNT: 0 no counters, kCountAll the counters of marches to the end of their
+// interval (fr_image.stats), kCountTaken those of the marches as the image kernels
+// take them, which end at the ball (fr_work_probe)
+constexpr int kCountAll = 1, kCountTaken = 2;
+
 // Sphere tracing (Listing "Julia Set ray cast"): from t0, d = DE(ro + t rd);
 // d < eps -> hit; t += min(d, max_step); t > t1 -> miss; running out of steps
 // inside the interval is reported as a hit at the current t.  The march ends as
 // a miss as soon as the ray has left the fractal's ball (exit_t) with steps
 // enough in hand to reach t1: the same outcome, without the distances on the
-// way out (the counting kernels take them, for their counters).  One condition
-// ends the loop (see the whole-orbit DEs).
-template <int KIND, int U, bool COUNT>
+// way out (kCountAll takes them, for its counters).  One condition ends the loop
+// (see the whole-orbit DEs).
+template <int KIND, int U, int COUNT>
 __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, float t0, float t1,
                                       float &t_out, int &steps_out, Counters &cnt, int slot)
 {
@@ -23,7 +28,8 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
     int steps = 0;
     bool hit = true;
     float t_end = t1;
-    if (!COUNT) {
+    constexpr bool to_end = COUNT == kCountAll;
+    if (!to_end) {
         t_end = exit_t(R, ro, rd, t1);
         if (t > t_end) {
             if (R.exit_steps <= R.max_steps) return false;
@@ -44,7 +50,7 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
             going = on && hit && steps < R.max_steps;
         } while (going);
         // out of the ball too close to the step cap: on to t1 itself
-        if (COUNT || hit || t > t1 || steps + R.exit_steps <= R.max_steps) break;
+        if (to_end || hit || t > t1 || steps + R.exit_steps <= R.max_steps) break;
         if (steps == R.max_steps) {
             hit = true;
             break;
@@ -67,7 +73,7 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
 // it slowed the Phong frame by 7 % (instruction fetch).  BAN 1 inlines it (the
 // single-request kernels for such requests), BAN 2 calls it out of line (the
 // batch kernels, which carry it for every launch).
-template <int KIND, int U, bool COUNT, int BAN>
+template <int KIND, int U, int COUNT, int BAN>
 __device__ __forceinline__ float3 normal_at(const DevReq &R, float3 x, float3 rd, Counters &cnt)
 {
     if ((KIND == 0 || BAN) && R.normal_mode == 2) {
@@ -106,7 +112,7 @@ __device__ __forceinline__ float3 normal_at(const DevReq &R, float3 x, float3 rd
 // single call site for all DE evaluations (one loop whose trips pick the point
 // by phase) measured slower again (1.10 ms; Julia 256^2 0.149 against
 // 0.117 ms): its phase bookkeeping costs more than the smaller code saves.
-template <int KIND, int U, bool COUNT, int BAN>
+template <int KIND, int U, int COUNT, int BAN>
 __device__ __forceinline__ float4 trace_sample(const DevReq &R, float3 ro, float3 rd, float &t_hit,
                                                uint32_t &flags, float3 &xhit, Counters &cnt)
 {
@@ -160,7 +166,7 @@ __device__ __forceinline__ float4 trace_sample(const DevReq &R, float3 ro, float
 // by Fresnel-Schlick in shade_phong.  The two hits' normals share one stencil
 // call, so the DE is still inlined twice.  Kept apart from the Lambert-only
 // loop above, which holds fewer live values.
-template <int KIND, int U, bool COUNT, int BAN>
+template <int KIND, int U, int COUNT, int BAN>
 __device__ __forceinline__ float4 trace_sample_phong(const DevReq &R, float3 ro, float3 rd, float &t_hit,
                                                      uint32_t &flags, float3 &xhit, Counters &cnt)
 {
@@ -233,7 +239,7 @@ __device__ __forceinline__ float4 trace_sample_phong(const DevReq &R, float3 ro,
 // warp's quad store (store_rgba8_depth).  PHONG compiles the Phong +
 // mirror-ray path in (requests still choose it with R.shading); without it the
 // Lambert-only code keeps fewer registers.
-template <int KIND, int U, bool COUNT, bool PHONG, int BAN = 0>
+template <int KIND, int U, int COUNT, bool PHONG, int BAN = 0>
 __device__ __forceinline__ void render_pixel(const DevReq &R, int px, int py, Counters &cnt, uint32_t &c8,
                                              float &depth)
 {
@@ -279,7 +285,7 @@ __device__ __forceinline__ void render_pixel(const DevReq &R, int px, int py, Co
 // give the same bits; its results are the pixel's.  `valid`: the pixel lies
 // inside the image.  (Kernels of their own: carried in the one-lane kernels,
 // this code cost the 1080p frame 2.5 %.)
-template <int KIND, int U, bool COUNT, bool PHONG, int BAN = 0>
+template <int KIND, int U, int COUNT, bool PHONG, int BAN = 0>
 __device__ __forceinline__ void render_pixel_lanes(const DevReq &R, int px, int py, int sample, bool valid,
                                                    Counters &cnt, uint32_t &c8, float &depth)
 {

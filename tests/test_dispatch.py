@@ -54,6 +54,7 @@ def test_kernel_scenes_reach_every_forward_kernel():
         for name, scenes, batch, tuning, stats in group():
             want = dict(rgba8=True, depth=True, stats=stats)
             reached.update(D.launches(scenes if batch else scenes[0], batch, tuning, **want))
-    forward = {k for k in D.kernels() if k[0] not in ("backward_kernel", "ffma_probe_kernel")}
+    probe = {("plain_kernel", (kind, 1, 2, 1, 1, 0)) for kind in (0, 1)}  # fr_work_probe's
+    forward = {k for k in D.kernels() if k[0] not in ("backward_kernel", "ffma_probe_kernel")} - probe
     assert reached <= forward
     assert reached == forward, sorted(forward - reached)
