@@ -31,10 +31,9 @@ __device__ __forceinline__ bool march(const DevReq &R, float3 ro, float3 rd, flo
     constexpr bool to_end = COUNT == kCountAll;
     if (!to_end) {
         t_end = exit_t(R, ro, rd, t1);
-        if (t > t_end) {
-            if (R.exit_steps <= R.max_steps) return false;
-            t_end = t1;
-        }
+        // set_exit gives no ball around which crossing the sphere could take more than
+        // half of max_steps
+        if (t > t_end) return false;
     }
     for (;;) {
         bool going;
