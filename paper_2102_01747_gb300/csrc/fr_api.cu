@@ -346,10 +346,14 @@ int lanes_per_pixel(const fr_tuning &tu, const fr::DevReq &R)
 // Lanes per pixel of a Lambert Mandelbulb image too small to fill the GPU: 2, 4
 // or 8, of which one works, while that leaves at most about three warps per
 // scheduler (608 of them).  A warp takes as long as its rays together at every
-// step, and with fewer rays it is done sooner: one ray per lane against the
-// choice here, 64x36 133 -> 115 us, 160x90 187 -> 181 us; at 320x180 (1840 warps)
-// 2 lanes per pixel still took 3 % off n = 8 but added 8 % to n = 3.  Phong images
-// and the Julia set's short steps gain nothing.
+// step, and with fewer rays it is done sooner, unless the lanes left idle cost more
+// issue slots than that wins.  One lane per pixel against the choice here, us, at 64x36,
+// 160x90 and 240x135 (frame 10 of the orbit): n = 8 107 -> 101, 177 -> 158, 185 -> 201;
+// trig-free 87 -> 83, 144 -> 128, 148 -> 156; with the analytic normal 107 -> 103, 183 -> 168,
+// 183 -> 207; n = 3 244 -> 234, 433 -> 384, 427 -> 408, analytic 284 -> 242, 504 -> 406,
+// 507 -> 439; n = 2 261 -> 275, 509 -> 593, 521 -> 566.  At 320x180 (1840 warps) 2 lanes per
+// pixel still took 3 % off n = 8 but added 8 % to n = 3.  Phong images and the Julia set's
+// short steps gain nothing.
 int idle_lanes(const fr::DevReq &R)
 {
     const long long warps = fr::plain_tiles(R);

@@ -60,11 +60,13 @@ cudaError_t launch_plain_wild(const DevReq &R, int block, cudaStream_t s);
 cudaError_t launch_batch_plain(const BatchArgs &A, long long ctas, int block, int unroll, bool count,
                                bool phong, cudaStream_t s);
 
-// the single-request kernel compiled with the Mandelbulb's analytic normal (unroll 1)
+// the single-request kernel compiled with the Mandelbulb's analytic normal (one unroll
+// depth for each shading and power)
 cudaError_t launch_plain_ban(const DevReq &R, int block, bool count, cudaStream_t s);
 
-// the one-ray-per-thread kernels with a pixel's samples on R.spl adjacent lanes
-// (unroll 1): one request, or a batch launch in which some request has spl > 1
+// the one-ray-per-thread kernels with a pixel's samples, or its one sample and spare
+// lanes, on R.spl adjacent lanes (one unroll depth each): one request, or a batch
+// launch in which some request has spl > 1
 cudaError_t launch_plain_lanes(const DevReq &R, int block, bool count, cudaStream_t s);
 cudaError_t launch_batch_plain_lanes(const BatchArgs &A, long long ctas, int block, bool count, bool phong,
                                      cudaStream_t s);

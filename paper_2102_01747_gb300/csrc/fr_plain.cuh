@@ -72,13 +72,14 @@ __device__ __forceinline__ void shade_tile(const DevReq &R, long long tile, Coun
 
 // BAN: compiled with the Mandelbulb's analytic normal (normal_at; 1 inline,
 // 2 out of line).
-// Register caps (at most 256 threads per block, as fr_set_tuning enforces):
-// given only the block size the compiler keeps to 73 registers and orders the
-// orbit step so that a warp waits on its own chain.  Measured at 64, 72, 80, 96
-// and 112 registers: the 1080p frame 0.69, 0.64, 0.61, 0.59, 0.60 ms, n = 6 at
-// 640x360 0.43, 0.41, 0.39, 0.37, 0.40, the 160x90 thumbnail 0.26, 0.21, 0.18,
-// 0.18, 0.18; Phong at 1080p 1.12, 1.04, 1.00, 0.98, 0.96 ms; 4K with 4 samples on
-// lanes 5.72, 5.66, 5.54, 5.59, 5.69.  The Julia set's kernels need 64.
+// Register caps (at most 256 threads per block, as fr_set_tuning enforces).  The cap
+// does more than the count that comes of it: with the block size given in its place
+// the power-8 kernel took 73 registers and the 1080p frame 0.625 ms, with the cap of 96 it
+// takes 74 and 0.59 ms.  Measured at 64, 72, 80, 96 and 112: the 1080p frame 0.69, 0.64,
+// 0.61, 0.59, 0.60 ms, n = 6 at 640x360 0.43, 0.41, 0.39, 0.37, 0.40, the 160x90 thumbnail
+// 0.26, 0.21, 0.18, 0.18, 0.18; Phong at 1080p 1.12, 1.04, 1.00, 0.98, 0.96 ms; 4K with 4
+// samples on lanes 5.72, 5.66, 5.54, 5.59, 5.69.  The Julia set's kernels take 64 to 68, with
+// Phong 75.
 template <bool PHONG, bool LANES>
 constexpr int plain_registers()
 {

@@ -2,10 +2,10 @@
 // pixel's 2, 4 or 8 samples on adjacent lanes (LANES, render_pixel_lanes), for
 // requests with R.spl > 1 (a translation unit of its own so that it compiles
 // in parallel with the rest).  Phong requests take the Phong-capable
-// instantiation, the Mandelbulb's analytic normal the BAN one, and Lambert
-// Mandelbulb requests of the power 8 one compiled for that power.  Unroll depth
-// 1 but for Lambert Mandelbulbs: power 8 with 2 samples at 1080p 1.00 ms rolled,
-// 0.96 at depth 2, 0.98 at 4 (4K with 4 samples 5.84, 5.66 ms), n = 4 with 4
+// instantiation, the Mandelbulb's analytic normal the BAN one, both at unroll depth 1,
+// and Lambert Mandelbulb requests of the power 8 with a stencil one compiled for that
+// power.  Depths of the stencil's Lambert Mandelbulbs: power 8 with 2 samples at 1080p
+// 1.00 ms rolled, 0.96 at depth 2, 0.98 at 4 (4K with 4 samples 5.84, 5.66 ms), n = 4 with 4
 // samples at 1283x723 1.64, 1.64, 1.56 ms.
 #include "fr_plain.cuh"
 
