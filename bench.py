@@ -28,20 +28,22 @@ sys.path.insert(0, ROOT)
 from paper_2102_01747_gb300 import workloads as W  # noqa: E402
 
 # FP32 operations per orbit iteration, the unit of work of the roofline's
-# achieved FLOP/s (units counted per step by the counting kernel).  Each figure
-# is the FP32 work the one-ray-per-thread kernel executes per orbit iteration,
-# everything included (orbit step, DE epilogue, march update, stencils, camera
-# ray, shading): ncu's SASS counters 2*FFMA + FADD + FMUL over one launch
-# divided by the iterations counted on the same scene (Mandelbulb n = 8 at
-# 1920x1080, the orbit loop unrolled 4 times: 7.363 G / 50.88 M = 144.7;
-# Julia p = 2 at 256x256: 356.3 M / 10.27 M = 34.7; Mandelbulb powers 2..10
-# at 960x540, the same scene and camera, one request each).  The degree-3
-# Julia figure is the degree-2 one scaled by the ratio of their orbit-step
-# arithmetic (28 / 24); Mandelbulb powers 11..16 take the n = 10 figure.
-FLOPS_PER_ITER = {("julia", 2): 34.7, ("julia", 3): 40.5,
-                  ("bulb", 2): 131.0, ("bulb", 3): 135.7, ("bulb", 4): 139.2, ("bulb", 5): 142.8,
-                  ("bulb", 6): 144.2, ("bulb", 7): 145.7, ("bulb", 8): 144.7, ("bulb", 9): 149.2,
-                  ("bulb", 10): 150.0}
+# achieved FLOP/s (units counted per step by fr_work_probe: the distances and
+# iterations that the image kernels evaluate).  Each figure is the FP32 work the
+# one-ray-per-thread kernel executes per orbit iteration, everything included
+# (orbit step, DE epilogue, march update, stencils, camera ray, shading): ncu's
+# SASS counters 2*FFMA + FADD + FMUL + 2*(2*FFMA2 + FADD2 + FMUL2) (a packed
+# instruction is two operations) over one launch divided by the iterations of
+# the same scene (Mandelbulb n = 8 at 1920x1080: 6.471 G / 44.41 M = 145.7; Julia
+# p = 2 at 3840x2160 with shadow rays: 40.49 G / 1109.9 M = 36.5, at 256x256, where four
+# steps per escape test compute some in vain, 41.0; Mandelbulb powers 2..10 at
+# 960x540, the same scene and camera, one request each).  The degree-3 Julia
+# figure is the degree-2 one scaled by the ratio of their orbit-step arithmetic
+# (28 / 24); Mandelbulb powers 11..16 take the n = 10 figure.
+FLOPS_PER_ITER = {("julia", 2): 36.5, ("julia", 3): 42.6,
+                  ("bulb", 2): 135.4, ("bulb", 3): 139.2, ("bulb", 4): 142.2, ("bulb", 5): 145.2,
+                  ("bulb", 6): 147.0, ("bulb", 7): 148.0, ("bulb", 8): 145.7, ("bulb", 9): 151.4,
+                  ("bulb", 10): 152.1}
 # The algorithmic count of the same work: the operations of the listings'
 # formulas as written, each math-library call (sqrt, pow, acos, atan2, sin,
 # cos, log) counted as one operation, nothing for the library's internals.
@@ -59,12 +61,12 @@ ALG_PER_DE = {"julia": 19, "bulb": 17}
 # configuration launches), from the ncu capture of the same command
 # (dram__bytes_read.sum + dram__bytes_write.sum); the frame's 16.6 MB of
 # stores are still in the 129 MB L2 when the kernel ends.
-TRAFFIC = {("bulb_1080p", "plain_kernel"): 58880 + 512}
+TRAFFIC = {("bulb_1080p", "plain_kernel"): 33280 + 512}
 # The kernel sources the two tables above were counted on (sha256 over these
 # files in this order): when the sources change, the bench reports the
 # figures as stale and the traffic as null until they are counted again.
 COUNTED_SOURCES = ("fr_device.cuh", "fr_math.cuh", "fr_trace.cuh", "fr_plain.cuh", "fr_plain.cu", "fr_launch.h")
-COUNTED_SHA = "273055e64402ef6e83b575aa52c654ab07f46c72ffc51245c32c84c13e18737b"
+COUNTED_SHA = "88e17d757f27b4f0acfb9c76548019ddfb61d09822893012e12e4954f090f588"
 FP32_LANES_PER_SM = 128  # FFMA lanes per SM (4 sub-partitions x 32), checked by the FFMA probe
 
 
