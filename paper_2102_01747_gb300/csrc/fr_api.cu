@@ -311,7 +311,8 @@ void set_exit(fr::DevReq &R)
                         : p == 2 ? 0.5 + std::sqrt(0.25 + C)
                                  : 1.0 + C / 2.0;  // r^3 - C >= r from here on
     // largest |z| and |z'| the kernels can meet outside the ball
-    const double top = std::fmax(std::fmax(std::sqrt((double)R.esc2), std::sqrt(bound * bound + (double)R.slice_w * R.slice_w)), 1.0);
+    const double far = std::sqrt(bound * bound + (double)R.slice_w * R.slice_w);
+    const double top = std::fmax(std::fmax(std::sqrt((double)R.esc2), far), 1.0);
     const double cmax = bulb ? bound : C;
     if (!((power(top, p) + cmax) < 1e15)) return;
     const double grow = std::log10(bulb ? p * power(top, p - 1) + 1.0 : p * p * power(top, 2 * (p - 1)));
